@@ -405,7 +405,7 @@ def run_ours(args):
                                         "bounds": "home +-1 rad, +-pi rad/s, +-10 rad/s^2, +-300 rad/s^3"}
         line["metric"] = line["metric"].replace("sample + rollout", "sample + QP projection + rollout")
         qa = qfl * K * sc.nu / (m["qp_ms"] * 1e-3) / 1e12
-        line["qp_projection"] = {"kernel": "qp_project_kernel", "ms": m["qp_ms"], "bound": "alu",
+        line["qp_projection"] = {"kernel": "qp_sample_kernel", "ms": m["qp_ms"], "bound": "alu",
                                  "flops_per_sequence": qfl, "achieved": qa, "peak": m["peak"],
                                  "unit": "TFLOP/s", "frac": qa / m["peak"]}
     if args.task is not None:

@@ -233,8 +233,8 @@ int mppi_best_controls(mppi_ctx *c, float *U_best, void *stream);
  *   scales   HOST, 4 floats > 0, or NULL for the MPPI_QP_SCALE_* defaults
  *   q0, qd0  device, n floats: each sequence's present position, velocity
  *   v_in     device, n x H; v_out device, n x H (may alias v_in)
- * 1 <= H <= MPPI_QP_MAX_H, iters >= 0, rho > 0, dt > 0.  Allocates a small
- * stream-ordered scratch block (cudaMallocAsync) per call. */
+ * 1 <= H <= MPPI_QP_MAX_H, iters >= 0, rho > 0, dt > 0.  One kernel launch;
+ * nothing is allocated or copied (the factors travel as its parameters). */
 int mppi_qp_project(int n, int H, float dt, const float *bounds, int iters, float rho, const float *scales,
                     const float *q0, const float *qd0, const float *v_in, float *v_out, void *stream);
 /* Turn the projection on inside the controller's iteration (iters > 0) or

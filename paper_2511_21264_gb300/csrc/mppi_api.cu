@@ -296,7 +296,8 @@ struct mppi_ctx {
     // QP smoothing projection (Eq. 5)
     int qp_iters = 0;
     float qp_dt = 0.0f;
-    void* d_qp = nullptr;  // nu QPClass records, then per joint the inverse (H <= 32) or 2H band rows
+    void* d_qp = nullptr;  // nu QPClass records, then qp_tabs tables (1, or one per joint)
+    int qp_tabs = 1;
     size_t qp_bytes = 0;
     // ball-task cost suite (Sec. IV-B)
     DevTask* d_task = nullptr;
@@ -713,21 +714,21 @@ static void drop_graph(mppi_ctx* c) {
     c->graph = nullptr;
 }
 
-// Projection launch: sequence i = j * K + k (a warp's sequences share a
-// joint, hence a band factor); output U[h][k][j] (h-major sample buffer).
+// Projection launch; output U[h][k][j] (h-major sample buffer).
 static int launch_projection(mppi_ctx* c, const float* state, const float* u_nom, cudaStream_t s) {
     const int na = c->m->info.na, nu = 2 * na, nq = 2 * na + 7;
-    const QPArgs q = qp_controller_args(nu, nq, c->K, c->H, c->qp_iters, c->qp_dt, c->d_qp, state, u_nom, c->d_sigma,
-                                        c->cov_sampling ? c->d_L : nullptr, c->seed, c->d_iter, c->d_U);
+    const QPArgs q = qp_controller_args(nu, nq, c->K, c->H, c->qp_iters, c->qp_dt, c->d_qp, c->qp_tabs, state, u_nom,
+                                        c->d_sigma, c->cov_sampling ? c->d_L : nullptr, c->seed, c->d_iter, c->d_U);
     return launch_qp(q, s);
 }
 
 }  // extern "C"
 
 namespace mppi {
-// Per-joint projection data of one controller: nu class records, then per
-// joint the dense inverse (H <= 32, warp kernel) or the band factor rows.
-int qp_build(int nu, int H, const float* bounds, float rho, const float* scales, std::vector<unsigned char>& host) {
+// Projection data of one controller: nu class records, then one table, or nu
+// of them when the joints' free row groups differ.
+int qp_build(int nu, int K, int H, const float* bounds, float rho, const float* scales,
+             std::vector<unsigned char>& host, int* n_tab) {
     static const float kDefault[4] = {MPPI_QP_SCALE_POSITION, MPPI_QP_SCALE_VELOCITY, MPPI_QP_SCALE_ACCELERATION,
                                       MPPI_QP_SCALE_JERK};
     const float* sc = scales ? scales : kDefault;
@@ -736,16 +737,20 @@ int qp_build(int nu, int H, const float* bounds, float rho, const float* scales,
         if (rc != MPPI_OK) return rc;
     }
     if (H > MPPI_QP_MAX_H) return MPPI_ERR_UNSUPPORTED;
-    const bool warp = H <= QP_WARP_MAX_H;
-    const size_t per = warp ? 32 * 32 * sizeof(float) : 2 * (size_t)H * sizeof(float4);
-    host.assign((size_t)nu * sizeof(QPClass) + (size_t)nu * per, 0);
-    QPClass* cls = reinterpret_cast<QPClass*>(host.data());
-    unsigned char* fac = host.data() + (size_t)nu * sizeof(QPClass);
+    const int L = qp_lanes(K * nu, H);
+    const size_t per = (size_t)qp_table_size(H, L) * sizeof(float4);
+    std::vector<QPClass> cls(nu);
+    *n_tab = 1;
     for (int j = 0; j < nu; ++j) {
         qp_make_class(bounds + 8 * j, sc, rho, &cls[j]);
+        if (std::memcmp(cls[j].s, cls[0].s, sizeof cls[0].s) != 0) *n_tab = nu;
+    }
+    host.assign((size_t)nu * sizeof(QPClass) + (size_t)*n_tab * per, 0);
+    std::memcpy(host.data(), cls.data(), (size_t)nu * sizeof(QPClass));
+    for (int j = 0; j < *n_tab; ++j) {
         const double scd[4] = {cls[j].s[0], cls[j].s[1], cls[j].s[2], cls[j].s[3]};
-        const int rc = warp ? qp_dense_inverse(H, rho, scd, reinterpret_cast<float*>(fac + j * per))
-                            : qp_band_factor(H, rho, scd, reinterpret_cast<float4*>(fac + j * per));
+        const int rc = qp_table(H, L, rho, scd,
+                                reinterpret_cast<float4*>(host.data() + (size_t)nu * sizeof(QPClass) + j * per));
         if (rc != MPPI_OK) return rc;
     }
     return MPPI_OK;
@@ -753,8 +758,8 @@ int qp_build(int nu, int H, const float* bounds, float rho, const float* scales,
 
 // Projection of the K x nu sampled sequences of one controller into its
 // h-major sample buffer U (Eq. 5).
-QPArgs qp_controller_args(int nu, int nq, int K, int H, int iters, float dt, const void* d_qp, const float* state,
-                          const float* u_nom, const float* sigma, const float* Lfac, uint64_t seed,
+QPArgs qp_controller_args(int nu, int nq, int K, int H, int iters, float dt, const void* d_qp, int n_tab,
+                          const float* state, const float* u_nom, const float* sigma, const float* Lfac, uint64_t seed,
                           const unsigned long long* iter_ptr, float* U) {
     QPArgs q{};
     q.n = K * nu;
@@ -762,14 +767,13 @@ QPArgs qp_controller_args(int nu, int nq, int K, int H, int iters, float dt, con
     q.iters = iters;
     q.per_cls = K;
     q.dt = dt;
+    q.L = qp_lanes(q.n, H);
+    q.tab_size = qp_table_size(H, q.L);
+    q.n_tab = n_tab;
     q.cls = static_cast<const QPClass*>(d_qp);
-    const unsigned char* fac = static_cast<const unsigned char*>(d_qp) + (size_t)nu * sizeof(QPClass);
-    if (H <= QP_WARP_MAX_H) q.minv = reinterpret_cast<const float*>(fac);
-    else q.band = reinterpret_cast<const float4*>(fac);
+    q.tab = reinterpret_cast<const float4*>(static_cast<const unsigned char*>(d_qp) + (size_t)nu * sizeof(QPClass));
     q.q0 = state;
     q.qd0 = state + nq;
-    q.q_per_seq = 0;
-    q.vin = nullptr;
     q.nu = nu;
     q.u_nom = u_nom;
     q.sigma = sigma;
@@ -777,11 +781,7 @@ QPArgs qp_controller_args(int nu, int nq, int K, int H, int iters, float dt, con
     q.seed = seed;
     q.iter_ptr = iter_ptr;
     q.out = U;
-    q.o_a = nu;                  // member k
-    q.o_b = 1;                   // class j
-    q.o_h = (long long)K * nu;   // step h
     q.n_cls = nu;
-    q.in_n = 0;
     q.out_n = (long long)H * K * nu;
     return q;
 }
@@ -799,7 +799,8 @@ int mppi_set_projection(mppi_ctx* c, const float* bounds, int iters, float rho, 
     if (!bounds) return MPPI_ERR_INVALID_ARG;
     const int nu = 2 * c->m->info.na;
     std::vector<unsigned char> host;
-    const int brc = qp_build(nu, c->H, bounds, rho, scales, host);
+    int n_tab = 1;
+    const int brc = qp_build(nu, c->K, c->H, bounds, rho, scales, host, &n_tab);
     if (brc != MPPI_OK) return brc;
     if (!c->d_U) return MPPI_ERR_UNSUPPORTED;
     const float dt = c->m->host.dt;
@@ -816,6 +817,7 @@ int mppi_set_projection(mppi_ctx* c, const float* bounds, int iters, float rho, 
     cudaError_t e = cudaMemcpy(c->d_qp, host.data(), bytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e);
     c->qp_iters = iters;
+    c->qp_tabs = n_tab;
     c->qp_dt = dt;
     drop_graph(c);  // a captured solve holds the old launches
     return MPPI_OK;

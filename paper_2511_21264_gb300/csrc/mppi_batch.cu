@@ -388,7 +388,8 @@ struct mppi_batch {
     std::vector<float*> d_eq8;       // Sigma, L (H x nu x nu each), then the elite indices
     std::vector<unsigned long long*> d_sel;
     std::vector<float*> d_Ubuf;      // H x K x nu projected samples
-    std::vector<void*> d_qp;         // projection classes and factors
+    std::vector<void*> d_qp;         // projection classes and tables
+    std::vector<int> qp_tabs;        // tables of each instance
     int qp_iters = 0;
     float qp_dt = 0.0f;
 };
@@ -446,8 +447,8 @@ int enqueue_batch(mppi_batch* b, cudaStream_t s) {
         const int nq = 2 * b->na + 7;
         for (int i = 0; i < b->n; ++i) {
             const BatchInst& I = b->inst[i];
-            const QPArgs q = qp_controller_args(b->nu, nq, I.K, I.H, b->qp_iters, b->qp_dt, b->d_qp[i], I.state, I.u,
-                                                I.sigma, I.cov_sampling ? I.Lfac : nullptr, I.seed, I.iter, I.U);
+            const QPArgs q = qp_controller_args(b->nu, nq, I.K, I.H, b->qp_iters, b->qp_dt, b->d_qp[i], b->qp_tabs[i],
+                                                I.state, I.u, I.sigma, I.cov_sampling ? I.Lfac : nullptr, I.seed, I.iter, I.U);
             const int rc = launch_qp(q, s);
             if (rc != MPPI_OK) return rc;
         }
@@ -603,6 +604,7 @@ int mppi_batch_create(const mppi_batch_desc* desc, int n, mppi_batch** out) {
     b->d_sel.assign(n, nullptr);
     b->d_Ubuf.assign(n, nullptr);
     b->d_qp.assign(n, nullptr);
+    b->qp_tabs.assign(n, 1);
     int rc = reshape(b);
     if (rc != MPPI_OK) {
         mppi_batch_destroy(b);
@@ -680,8 +682,10 @@ int mppi_batch_set_projection(mppi_batch* b, const float* bounds, int iters, flo
     if (!bounds) return MPPI_ERR_INVALID_ARG;
     const int nu = b->nu;
     std::vector<std::vector<unsigned char>> host(b->n);
+    std::vector<int> tabs(b->n);
     for (int i = 0; i < b->n; ++i) {
-        const int rc = qp_build(nu, b->inst[i].H, bounds + (size_t)i * nu * 8, rho, scales, host[i]);
+        const int rc = qp_build(nu, b->inst[i].K, b->inst[i].H, bounds + (size_t)i * nu * 8, rho, scales, host[i],
+                                &tabs[i]);
         if (rc != MPPI_OK) return rc;
     }
     float dt = 0.0f;
@@ -694,6 +698,7 @@ int mppi_batch_set_projection(mppi_batch* b, const float* bounds, int iters, flo
         BatchInst& I = b->inst[i];
         cudaFree(b->d_qp[i]);
         b->d_qp[i] = nullptr;
+        b->qp_tabs[i] = tabs[i];
         cudaError_t e = cudaMalloc(&b->d_qp[i], host[i].size());
         if (e == cudaSuccess) e = cudaMemcpy(b->d_qp[i], host[i].data(), host[i].size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess && !b->d_Ubuf[i])

@@ -154,19 +154,18 @@ struct QPClass {
     float pad[3];
 };
 
-// Arguments of the projection kernel (one thread per sequence).  Sequence i
-// belongs to class i / per_cls as member i % per_cls; element h of its input
-// and output sits at (member * a + class * b + h * h_stride).
+// Arguments of the projection kernels.  The controller form draws sequence
+// (sample k, joint j) itself and writes the h-major sample buffer; the
+// standalone form reads and writes n rows of H values.
 struct QPArgs {
-    int n, H, iters, per_cls;
+    int n, H, iters, per_cls;  // per_cls: samples K (controller form, n = K nu)
     float dt;
-    const QPClass* cls;  // classes
-    const float4* band;  // per class 2H: forward then backward band factor rows
-    const float* q0;     // present position, per sequence (q_per_seq) or per class
-    const float* qd0;    // present velocity, same indexing
-    int q_per_seq;
-    const float* vin;    // explicit input, or null to sample (member = sample k, class = joint j)
-    long long i_a, i_b, i_h;
+    int L, tab_size, n_tab;    // lanes per sequence, float4s of a table, tables (1: shared by all joints)
+    const QPClass* cls;        // classes, one per joint
+    const float4* tab;         // tables
+    const float* q0;           // present position, per sequence or per joint
+    const float* qd0;          // present velocity, same indexing
+    const float* vin;          // standalone input
     // sampling: v = u_nom[h, j] + sigma_j z_j, or + (L_h z)_j with Lfac (no clamp)
     int nu;
     const float* u_nom;
@@ -176,21 +175,20 @@ struct QPArgs {
     const unsigned long long* iter_ptr;
     unsigned long long iter_val;
     float* out;
-    long long o_a, o_b, o_h;
-    const float* minv;   // H <= 32: per class the 32 x 32 inverse (I + rho D^T D)^-1 in velocity coordinates
     // extents, for the bounds-check build: classes, floats of vin and of out
     int n_cls;
     long long in_n, out_n;
 };
-constexpr int QP_WARP_MAX_H = 32;
-int qp_band_factor(int H, double rho, const double sc[4], float4* band);
-int qp_dense_inverse(int H, double rho, const double sc[4], float* minv);
+int qp_lanes(int n, int H);
+int qp_table_size(int H, int L);
+int qp_table(int H, int L, double rho, const double sc[4], float4* out);
 void qp_make_class(const float b[8], const float sc[4], float rho, QPClass* c);
 int qp_validate(const float b[8], const float sc[4], float rho);
 int launch_qp(const QPArgs& a, cudaStream_t s);
-int qp_build(int nu, int H, const float* bounds, float rho, const float* scales, std::vector<unsigned char>& host);
-QPArgs qp_controller_args(int nu, int nq, int K, int H, int iters, float dt, const void* d_qp, const float* state,
-                          const float* u_nom, const float* sigma, const float* Lfac, uint64_t seed,
+int qp_build(int nu, int K, int H, const float* bounds, float rho, const float* scales,
+             std::vector<unsigned char>& host, int* n_tab);
+QPArgs qp_controller_args(int nu, int nq, int K, int H, int iters, float dt, const void* d_qp, int n_tab,
+                          const float* state, const float* u_nom, const float* sigma, const float* Lfac, uint64_t seed,
                           const unsigned long long* iter_ptr, float* U);
 
 // closed-loop episode helpers

@@ -58,7 +58,8 @@ struct Scene {
     float eta = 1.0f, cov_floor = 0.0f;
     float* d_eq8 = nullptr;              // Sigma, L (H x nu x nu each), elite indices (K)
     unsigned long long* d_sel = nullptr;
-    void* d_qp = nullptr;                // projection classes and factors (server-wide projection)
+    void* d_qp = nullptr;                // projection classes and tables (server-wide projection)
+    int qp_tabs = 1;
 };
 
 struct Request {
@@ -288,8 +289,8 @@ int launch_lane(mppi_server* S, Lane& ln) {
         const BatchInst& I = ln.h_insts[e];
         const Scene& sc = S->scenes[act[e]->scene];
         const QPArgs q = qp_controller_args(sc.nu, 2 * S->na + 7, sc.K, sc.H, S->cfg.qp_iters, model_dt(sc.model),
-                                            sc.d_qp, I.state, I.u, I.sigma, I.cov_sampling ? I.Lfac : nullptr, I.seed,
-                                            I.iter, I.U);
+                                            sc.d_qp, sc.qp_tabs, I.state, I.u, I.sigma, I.cov_sampling ? I.Lfac : nullptr,
+                                            I.seed, I.iter, I.U);
         rc = launch_qp(q, ln.stream);
     }
     if (rc == MPPI_OK) rc = launch_batch_iteration(ln.d_insts, n, t, row, ln.d_ctl, L, ln.stream);
@@ -616,10 +617,12 @@ int srv_set_scene_projection(mppi_server* S, int scene_id, const float* bounds, 
         return MPPI_ERR_INVALID_ARG;
     Scene& sc = S->scenes[scene_id];
     std::vector<unsigned char> host;
-    const int rc = qp_build(sc.nu, sc.H, bounds, rho, scales, host);
+    int n_tab = 1;
+    const int rc = qp_build(sc.nu, sc.K, sc.H, bounds, rho, scales, host, &n_tab);
     if (rc != MPPI_OK) return rc;
     cudaFree(sc.d_qp);
     sc.d_qp = nullptr;
+    sc.qp_tabs = n_tab;
     cudaError_t e = cudaMalloc(&sc.d_qp, host.size());
     if (e == cudaSuccess) e = cudaMemcpy(sc.d_qp, host.data(), host.size(), cudaMemcpyHostToDevice);
     return cuda_rc(e);
