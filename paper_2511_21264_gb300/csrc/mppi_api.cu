@@ -196,6 +196,10 @@ int parse_model_blob(const void* blob, size_t len, DevModel* out, HostModelInfo*
     M.w_grasp = (float)v(22);
     if (!(M.dt > 0) || M.sweeps < 0 || M.sweeps > 1000 || !(M.imp > 0 && M.imp <= 1) || !(M.mb > 0) || !(M.Ib > 0))
         return MPPI_ERR_INVALID_ARG;
+    M.im = 1.0f / M.mb;
+    M.iI = 1.0f / M.Ib;
+    M.regc = (1.0f - M.imp) / M.imp;
+    M.erp_dt = M.erp / M.dt;
     size_t o = 23;
     for (int a = 0; a < 2; ++a) {
         for (int k = 0; k < 9; ++k) M.baseR[a][k] = (float)v(o++);

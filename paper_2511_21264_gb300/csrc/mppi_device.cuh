@@ -63,6 +63,7 @@ struct __align__(16) DevModel {
     CArr<float, 3> g;
     float floor_z;
     float rb, mb, Ib, pad0;
+    float im, iI, regc, erp_dt;  // 1/mb, 1/Ib, (1 - imp)/imp, erp/dt
     CArr<float, 3> goal;
     float w_goal;
     float w_u, w_pen, w_obst, w_grasp;
@@ -111,6 +112,7 @@ struct Lanes {
     __device__ __forceinline__ int xor_(int v, int off) const { return __shfl_xor_sync(gm, v, off, LPS); }
     // within the lane's arm segment
     __device__ __forceinline__ float up_seg(float v, int off) const { return __shfl_up_sync(gm, v, off, SEG); }
+    __device__ __forceinline__ float from_seg(float v, int src) const { return __shfl_sync(gm, v, src, SEG); }
     __device__ __forceinline__ float down_seg(float v, int off) const { return __shfl_down_sync(gm, v, off, SEG); }
 };
 
@@ -171,11 +173,11 @@ struct __align__(16) WarpWS {
             CArr<short, 2 * MAXL * MAXB> surv;  // capsule-box pairs that pass the cull
         } col;
         struct {
-            CArr<CArr<float, d::NV>, MAXR> Y;
-            CArr<float, MAXR * MAXR> G;  // Delassus block Y Y^T, nr x nr
-            CArr<float4, MAXR> rc4;      // per row: b = J v_f, R, 1/(A+R), reference velocity
+            CArr<CArr<float4, (d::NV + 3) / 4>, MAXR> Y;  // half-solved rows, zero-padded to whole float4s
+            CArr<float, 9 * MAXC * MAXC> G;  // Delassus entry (3 c + k, 3 q + m) at ((9 q + 3 k + m) MAXC + c), R added on the diagonal
+            CArr<float, MAXR> rho;       // per row: b - reference velocity, with b = J v_f
+            CArr<float, MAXR> iA;        // 1 / (A + R)
             CArr<float, MAXR> lam;
-            CArr<int, MAXR> tmask;       // blocks a row touches: 1 left arm, 2 right arm, 4 ball
         } con;
     } ph;
 };
@@ -291,16 +293,21 @@ __device__ __forceinline__ void forward_kinematics(const DevModel& M, WarpWS<NA>
         p[1] = sn * L.Fp[0] + cs * L.Fp[1];
         p[2] = L.Fp[2];
     }
+    // the lanes past the last link hold the identity through all rounds, and a
+    // lane with no predecessor this far back takes it from there: no selects
+    // on the products (24 of about 2,000 instructions of a step)
+#pragma unroll
+    for (int k = 0; k < 9; ++k) R[k] = act ? R[k] : (k % 4 == 0 ? 1.0f : 0.0f);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) p[k] = act ? p[k] : 0.0f;
 #pragma unroll
     for (int off = 1; off < NA; off <<= 1) {
+        const int src = act && i >= off ? i - off : NA;
         float Rp[9], pp[3];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) Rp[k] = g.up_seg(R[k], off);
+        for (int k = 0; k < 9; ++k) Rp[k] = g.from_seg(R[k], src);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) pp[k] = g.up_seg(p[k], off);
-        // every lane forms the product; lanes with no predecessor this far
-        // back keep their transform (a select, no divergent branch)
-        const bool take = i >= off;
+        for (int k = 0; k < 3; ++k) pp[k] = g.from_seg(p[k], src);
         float Rn[9], pn[3];
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
@@ -310,9 +317,9 @@ __device__ __forceinline__ void forward_kinematics(const DevModel& M, WarpWS<NA>
             pn[r] = Rp[3 * r] * p[0] + Rp[3 * r + 1] * p[1] + Rp[3 * r + 2] * p[2] + pp[r];
         }
 #pragma unroll
-        for (int k = 0; k < 9; ++k) R[k] = take ? Rn[k] : R[k];
+        for (int k = 0; k < 9; ++k) R[k] = Rn[k];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) p[k] = take ? pn[k] : p[k];
+        for (int k = 0; k < 3; ++k) p[k] = pn[k];
     }
     // world frame: base * chain
     const float* B = M.baseR[a];
@@ -534,12 +541,14 @@ __device__ __forceinline__ float capsule_box_candidate(int id, const float* a, c
 // Ball pairs live in 32 fixed slots: slot 0 the floor, slot 1 + l link l
 // (l < 2 n_a <= 14), slot 16 + b box b (b < 16); slot t sits on group lane
 // t % LPS as element t / LPS of the lane's depth sums.  One pass covers the
-// LPS slots of one element: a pass that holds floor and link slots only runs
-// the capsule test, one that holds box slots only runs the box test, and the
-// single pass of a 32-lane group (both kinds) runs both tests on every lane
-// and keeps the one its slot needs -- no divergent branches.  Contacts are
-// compacted with a ballot per pass, in slot order, which is the canonical
-// pair order.
+// LPS slots of one element.  Every lane forms the squared distance that its
+// slot needs; the signed distance, normal and contact point of the links and
+// boxes only follow where some pair of the group comes near (the ball is
+// clear of them on most steps), with the contacts compacted by a ballot in
+// slot order, which is the canonical pair order.  The floor, slot 0, is
+// tested by every lane (it is the first contact when it is one).  Normals and
+// points on every step, as before, with the floor's solve in its general form:
+// transfer iteration (K = 4096, H = 64) 366 us, lift 115; so 342 and 108.
 template <int NA, int LPS, int S>
 __device__ __forceinline__ void ball_pass(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g,
                                           float (&pa)[32 / LPS], float (&pbox)[32 / LPS], int& base,
@@ -554,38 +563,53 @@ __device__ __forceinline__ void ball_pass(const DevModel& M, WarpWS<NA>& w, cons
     const int slot = lo + g.sl;
     const float* pb = &w.q[d::B];
     const float rb = M.rb;
-    const bool isf = slot == 0, isc = slot >= 1 && slot <= d::NL, isb = slot >= 16 && slot < 16 + nb;
-    float dist = 1.0f, nn[3] = {0.0f, 0.0f, 1.0f}, cp[3] = {0.0f, 0.0f, 0.0f};
+    const bool isc = slot >= 1 && slot <= d::NL, isb = slot >= 16 && slot < 16 + nb;
+    constexpr float slack = 1e-3f;  // m; the squared distances are compared with a margin far above their rounding
+    bool near = false;
     const int l = min(max(slot - 1, 0), d::NL - 1);
-    if constexpr (has_link) {  // ball - capsule, and the floor on slot 0
+    const float rc = M.link[l / NA][l % NA].rcap;
+    float sp[3], df[3], d2 = 0.0f;
+    if constexpr (has_link) {  // ball - capsule: closest point of the segment
         const float* a0 = w.a0[l];
         const float* a1 = w.a1[l];
-        float dd[3] = {a1[0] - a0[0], a1[1] - a0[1], a1[2] - a0[2]};
-        float ac[3] = {pb[0] - a0[0], pb[1] - a0[1], pb[2] - a0[2]};
+        const float dd[3] = {a1[0] - a0[0], a1[1] - a0[1], a1[2] - a0[2]};
+        const float ac[3] = {pb[0] - a0[0], pb[1] - a0[1], pb[2] - a0[2]};
         const float den = dot3(dd, dd);
         float t = den > 0.0f ? dot3(ac, dd) / den : 0.0f;
         t = fminf(fmaxf(t, 0.0f), 1.0f);
-        float sp[3] = {a0[0] + t * dd[0], a0[1] + t * dd[1], a0[2] + t * dd[2]};
-        float df[3] = {pb[0] - sp[0], pb[1] - sp[1], pb[2] - sp[2]};
-        const float len = sqrtf(dot3(df, df));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            sp[k] = a0[k] + t * dd[k];
+            df[k] = pb[k] - sp[k];
+        }
+        d2 = dot3(df, df);
+        near = isc && d2 <= (rb + rc + slack) * (rb + rc + slack);
+    }
+    const float* box = M.box[nb > 0 ? min(max(slot - 16, 0), nb - 1) : 0];
+    if constexpr (has_box) {  // ball - box: the part of the centre's offset outside the box
+        if (nb > 0) {
+            float q2 = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float e = fmaxf(fabsf(pb[k] - box[k]) - box[3 + k], 0.0f);
+                q2 = __fmaf_rn(e, e, q2);
+            }
+            near = near || (isb && q2 <= (rb + slack) * (rb + slack));
+        }
+    }
+    if (!g.any(near)) return;
+    float dist = 1.0f, nn[3] = {0.0f, 0.0f, 1.0f}, cp[3] = {0.0f, 0.0f, 0.0f};
+    if constexpr (has_link) {
+        const float len = sqrtf(d2);
         const float il = 1.0f / len;
-        nn[0] = !isf && len > 0.0f ? df[0] * il : 0.0f;
-        nn[1] = !isf && len > 0.0f ? df[1] * il : 0.0f;
-        nn[2] = !isf && len > 0.0f ? df[2] * il : 1.0f;
-        const float rc = M.link[l / NA][l % NA].rcap;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) nn[k] = len > 0.0f ? df[k] * il : (k == 2 ? 1.0f : 0.0f);
 #pragma unroll
         for (int k = 0; k < 3; ++k) cp[k] = 0.5f * ((pb[k] - rb * nn[k]) + (sp[k] + rc * nn[k]));
         dist = len - rb - rc;
-        if (isf) {  // ball - floor
-            dist = (pb[2] - M.floor_z) - rb;
-            cp[0] = pb[0];
-            cp[1] = pb[1];
-            cp[2] = 0.5f * ((pb[2] - rb) + M.floor_z);
-        }
     }
-    if constexpr (has_box) {  // ball - box
+    if constexpr (has_box) {
         if (nb > 0) {
-            const float* box = M.box[min(max(slot - 16, 0), nb - 1)];
             float nb3[3], surf[3];
             const float db = box_sdf(pb, box, nb3, surf) - rb;
             if (isb) {
@@ -599,7 +623,7 @@ __device__ __forceinline__ void ball_pass(const DevModel& M, WarpWS<NA>& w, cons
         }
     }
     const int Bb = isc ? l : -1;
-    const bool active = (isf || isc || isb) && dist < 0.0f;
+    const bool active = (isc || isb) && dist < 0.0f;
     const unsigned mask = g.ballot(active);
     const int pos = base + __popc(mask & ((1u << g.sl) - 1u));
     const bool keep = active && pos < M.maxc;
@@ -622,25 +646,41 @@ __device__ __forceinline__ void ball_pass(const DevModel& M, WarpWS<NA>& w, cons
 // Narrow phase in canonical pair order (ball-floor, ball-links, ball-boxes,
 // links x boxes).  Ball pairs: one lane per pair slot (above), exact,
 // compacted with a ballot.  Capsule-box pairs: a conservative
-// separating-axis cull per lane (segment_meets_inflated_box), then each
-// surviving pair (in pair order) is minimised by the whole group over the
-// candidate set above.  Each lane adds
+// separating-axis cull per lane (segment_meets_inflated_box), here; each
+// surviving pair (in pair order) is then minimised by the whole group over the
+// candidate set above, in collide_exact.  Each lane adds
 // the depths of the contacts it found to pa (all) and pbox (against boxes),
-// per slot element; every lane gets the number of stored contacts (ncon) and
-// the blocks they touch (tb: 1 left arm, 2 right arm, 4 ball).  Returns the
-// number of exact capsule-box tests on group lane 0 (0 on the other lanes).
+// per slot element.
+struct Contacts {
+    int base = 0;         // active contacts so far (stored up to the cap)
+    int nsurv = 0;        // capsule-box pairs that passed the cull
+    unsigned tbits = 0u;  // blocks this lane's stored contacts touch
+    int ncon, tb;         // stored contacts; the blocks they touch (1 left arm, 2 right arm, 4 ball)
+    float floor = -1.0f;  // depth of the ball in the floor (the first contact) when positive
+    template <int LPS>
+    __device__ __forceinline__ void close(const DevModel& M, const Lanes<LPS>& g) {
+        tb = (int)__reduce_or_sync(g.gm, tbits);
+        ncon = base < M.maxc ? base : M.maxc;
+    }
+};
 template <int NA, int LPS>
-__device__ __forceinline__ int collide(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g,
-                                      float (&pa)[32 / LPS], float (&pbox)[32 / LPS], int& ncon, int& tb) {
+__device__ __forceinline__ void collide(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g,
+                                        float (&pa)[32 / LPS], float (&pbox)[32 / LPS], Contacts& con) {
     using d = Dims<NA>;
     const int nb = M.nb;
-    int base = 0, nsurv = 0;
-    unsigned tbits = 0u;  // blocks the stored contacts touch
-    ball_pass<NA, LPS, 0>(M, w, g, pa, pbox, base, tbits);
-    if constexpr (LPS <= 16) ball_pass<NA, LPS, 1>(M, w, g, pa, pbox, base, tbits);
+    {  // ball - floor, on every lane; stored by store_floor where a solve reads it
+        const float dist = (w.q[d::B + 2] - M.floor_z) - M.rb;
+        const bool active = dist < 0.0f;
+        con.floor = -dist;
+        con.base = active ? 1 : 0;
+        con.tbits = active ? 4u : 0u;
+        pa[0] += active && g.sl == 0 ? -dist : 0.0f;
+    }
+    ball_pass<NA, LPS, 0>(M, w, g, pa, pbox, con.base, con.tbits);
+    if constexpr (LPS <= 16) ball_pass<NA, LPS, 1>(M, w, g, pa, pbox, con.base, con.tbits);
     if constexpr (LPS <= 8) {
-        ball_pass<NA, LPS, 2>(M, w, g, pa, pbox, base, tbits);
-        ball_pass<NA, LPS, 3>(M, w, g, pa, pbox, base, tbits);
+        ball_pass<NA, LPS, 2>(M, w, g, pa, pbox, con.base, con.tbits);
+        ball_pass<NA, LPS, 3>(M, w, g, pa, pbox, con.base, con.tbits);
     }
     // capsule-box: lane l (and, where a pass over the links fills half the
     // group, lane CL + l) tests link l's capsule against the boxes (or one
@@ -670,22 +710,32 @@ __device__ __forceinline__ int collide(const DevModel& M, WarpWS<NA>& w, const L
         }
         const int cnt = __popc(smask);
         const int cnt_link = NH == 2 ? cnt + g.xor_(cnt, CL) : cnt;  // both halves of link l
-        int pre = cnt_link;  // inclusive prefix over the links (both halves alike)
+        if (g.any(smask != 0u)) {
+            int pre = cnt_link;  // inclusive prefix over the links (both halves alike)
 #pragma unroll
-        for (int off = 1; off < CL; off <<= 1) {
-            const int o = __shfl_up_sync(g.gm, pre, off, CL);
-            if (l >= off) pre += o;
+            for (int off = 1; off < CL; off <<= 1) {
+                const int o = __shfl_up_sync(g.gm, pre, off, CL);
+                if (l >= off) pre += o;
+            }
+            int pos = pre - cnt_link + (half ? cnt_link - cnt : 0);
+            while (smask) {
+                const int bi = __ffs(smask) - 1;
+                smask &= smask - 1u;
+                w.ph.col.surv[pos++] = (short)(l * nb + bi);
+            }
+            con.nsurv = g.shfl(pre, CL - 1);
         }
-        int pos = pre - cnt_link + (half ? cnt_link - cnt : 0);
-        while (smask) {
-            const int bi = __ffs(smask) - 1;
-            smask &= smask - 1u;
-            w.ph.col.surv[pos++] = (short)(l * nb + bi);
-        }
-        nsurv = g.shfl(pre, CL - 1);
     }
-    g.sync();
-    for (int si = 0; si < nsurv; ++si) {
+    con.close(M, g);
+}
+
+// The exact test of the pairs that passed the cull.
+template <int NA, int LPS>
+__device__ __forceinline__ void collide_exact(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g,
+                                              float (&pa)[32 / LPS], float (&pbox)[32 / LPS], Contacts& con) {
+    const int nb = M.nb;
+    int& base = con.base;
+    for (int si = 0; si < con.nsurv; ++si) {
         const int idx = w.ph.col.surv[si];
         const int l = idx / nb, bi = idx - l * nb;
         const float* box = M.box[bi];
@@ -720,7 +770,7 @@ __device__ __forceinline__ int collide(const DevModel& M, WarpWS<NA>& w, const L
                 pa[0] += -dist;
                 pbox[0] += -dist;
                 if (base < M.maxc) {
-                    tbits |= 1u << (l / NA);
+                    con.tbits |= 1u << (l / NA);
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         w.cp[base][k] = 0.5f * ((x[k] - rc * nn[k]) + surf[k]);
@@ -734,9 +784,7 @@ __device__ __forceinline__ int collide(const DevModel& M, WarpWS<NA>& w, const L
             ++base;
         }
     }
-    tb = (int)__reduce_or_sync(g.gm, tbits);
-    ncon = base < M.maxc ? base : M.maxc;
-    return g.sl == 0 ? nsurv : 0;
+    con.close(M, g);
 }
 
 // ---------------------------------------------------------------------------
@@ -1043,7 +1091,7 @@ __device__ __forceinline__ void ball_contact_dv(const DevModel& M, const WarpWS<
                                                 const float* va, float (&dv)[6]) {
     using d = Dims<NA>;
     constexpr int NR = 3 * NC;
-    const float im = 1.0f / M.mb, iI = 1.0f / M.Ib, regc = (1.0f - M.imp) / M.imp;
+    const float im = M.im, iI = M.iI, regc = M.regc;
     const float* bc = &w.q[d::B];
     // rows without the side sign s_c (+1 when the ball is body A): it enters
     // b, the cross-contact Delassus entries and the applied impulse
@@ -1072,7 +1120,7 @@ __device__ __forceinline__ void ball_contact_dv(const DevModel& M, const WarpWS<
                 D[r][q] = de[q];
             }
             bb[r] = sgn * (dot3(E[r], vl) + dot3(D[r], va));
-            vs[r] = k == 0 ? (M.erp / M.dt) * w.cdep[c] : 0.0f;
+            vs[r] = k == 0 ? M.erp_dt * w.cdep[c] : 0.0f;
         }
     }
     float G[NR][NR], R[NR], iA[NR], lam[NR];
@@ -1172,12 +1220,70 @@ __device__ __forceinline__ void ball_contact_dv(const DevModel& M, const WarpWS<
     }
 }
 
+// The same for the lone contact with the floor (depth dep): normal (0, 0, 1),
+// tangents (0, 1, 0) and (-1, 0, 0) as contact_frame_row gives them, lever arm
+// (0, 0, dz), so that every row is a component of the ball's velocity and one
+// product.
+template <int NA>
+__device__ __forceinline__ void floor_contact_dv(const DevModel& M, const WarpWS<NA>& w, const float* vl,
+                                                 const float* va, float dep, float (&dv)[6]) {
+    using d = Dims<NA>;
+    const float bz = w.q[d::B + 2];
+    const float dz = 0.5f * ((bz - M.rb) + M.floor_z) - bz;
+    const float gn = M.im, gt = __fmaf_rn(M.iI, __fmul_rn(dz, dz), M.im);
+    const float in = 1.0f / __fmaf_rn(M.regc, gn, gn), it = 1.0f / __fmaf_rn(M.regc, gt, gt);
+    float ln = 0.0f, l1 = 0.0f, l2 = 0.0f;
+    if (M.sweeps > 0) {
+        ln = fmaxf(__fmaf_rn(M.erp_dt, dep, -vl[2]) * in, 0.0f);
+        l1 = -__fmaf_rn(-dz, va[0], vl[1]) * it;
+        l2 = __fmaf_rn(dz, va[1], vl[0]) * it;
+        const float n2 = __fmaf_rn(l1, l1, __fmul_rn(l2, l2)), lim = M.mu * ln;
+        const float sc = n2 > lim * lim ? lim * rsqrtf(n2) : 1.0f;
+        l1 *= sc;
+        l2 *= sc;
+    }
+    const float gd = -M.iI * dz;
+    dv[0] = -M.im * l2;
+    dv[1] = M.im * l1;
+    dv[2] = M.im * ln;
+    dv[3] = gd * l1;
+    dv[4] = gd * l2;
+    dv[5] = 0.0f;
+}
+
+// A lone ball contact with static geometry: the floor's (floor > 0, its depth)
+// or the stored one.
+template <int NA>
+__device__ __forceinline__ void lone_contact_dv(const DevModel& M, const WarpWS<NA>& w, const float* vl,
+                                                const float* va, float floor, float (&dv)[6]) {
+    if (floor > 0.0f) floor_contact_dv<NA>(M, w, vl, va, floor, dv);
+    else ball_contact_dv<NA, 1, 0>(M, w, vl, va, dv);
+}
+
+// The floor's contact record, slot 0 of the step's contacts.
+template <int NA, int LPS>
+__device__ __forceinline__ void store_floor(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g, float floor) {
+    using d = Dims<NA>;
+    if (floor > 0.0f && g.sl == 0) {
+        const float* pb = &w.q[d::B];
+        w.cp[0][0] = pb[0];
+        w.cp[0][1] = pb[1];
+        w.cp[0][2] = 0.5f * ((pb[2] - M.rb) + M.floor_z);
+        w.cn[0][0] = w.cn[0][1] = 0.0f;
+        w.cn[0][2] = 1.0f;
+        w.cdep[0] = floor;
+        w.cA[0] = d::B;
+        w.cB[0] = -1;
+    }
+}
+
 // v = v_f + M^-1 J^T lambda on the ball, v_f elsewhere.
 template <int NA, int NC, int LPS>
-__device__ __forceinline__ void contacts_ball(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g) {
+__device__ __forceinline__ void contacts_ball(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g, float floor) {
     using d = Dims<NA>;
     float dv[6];
-    ball_contact_dv<NA, NC, 0>(M, w, &w.vf[d::B], &w.vf[d::B + 3], dv);
+    if constexpr (NC == 1) lone_contact_dv<NA>(M, w, &w.vf[d::B], &w.vf[d::B + 3], floor, dv);
+    else ball_contact_dv<NA, NC, 0>(M, w, &w.vf[d::B], &w.vf[d::B + 3], dv);
 #pragma unroll
     for (int c0 = 0; c0 < d::NV; c0 += LPS) {
         const int c = c0 + g.sl;
@@ -1192,16 +1298,16 @@ __device__ __forceinline__ void contacts_ball(const DevModel& M, WarpWS<NA>& w, 
     g.sync();
 }
 
-// The free velocity and a ball-only contact solve together (one or two
-// contacts of the ball with static geometry; SW sweeps for two).  Every lane of an
+// The free velocity and the lone contact of the ball with static geometry
+// together.  Every lane of an
 // arm's half-warp factors that arm's block and solves for its free velocity
 // (the operations of the one-lane factor in dynamics) while every lane runs
 // the contact solve: with no divergence between them the two independent
 // chains share the issue slots.  Writes v: the arms' free velocities and the
 // ball's after the impulses (the values dynamics and contacts_ball give).
-template <int NA, int NC, int SW, int LPS>
-__device__ __forceinline__ void solve_ball_contacts(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g,
-                                                    int* err) {
+template <int NA, int LPS>
+__device__ __forceinline__ void solve_ball_contact(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g, int* err,
+                                                   float floor) {
     using d = Dims<NA>;
     constexpr int SEG = Lanes<LPS>::SEG;
     const int a = g.a, i = g.i;
@@ -1215,7 +1321,7 @@ __device__ __forceinline__ void solve_ball_contacts(const DevModel& M, WarpWS<NA
     bool ok;
     arm_solve<NA>(w, a, A, di, y, ok);
     float dv[6];
-    ball_contact_dv<NA, NC, SW>(M, w, vb, vb + 3, dv);
+    lone_contact_dv<NA>(M, w, vb, vb + 3, floor, dv);
     if (i == 0 && !ok) atomicOr(err, ERRB_CHOLESKY);
     // lane i < NA of segment a: the arm's velocity i (formed on every lane,
     // one stored); the ball's lane stores the ball's six
@@ -1232,57 +1338,76 @@ __device__ __forceinline__ void solve_ball_contacts(const DevModel& M, WarpWS<NA
     g.sync();
 }
 
-// Projected Gauss-Seidel for one or two contacts with the Delassus block in
-// registers: every lane runs the same sweeps (no shuffles, no shared-memory
-// round trips), then lane r stores lambda_r.  The same iteration as the
-// lane-parallel path below, summed in a different order.
+// v = v_f: no contact
+template <int NA, int LPS>
+__device__ __forceinline__ void free_velocity(WarpWS<NA>& w, const Lanes<LPS>& g) {
+    using d = Dims<NA>;
+#pragma unroll
+    for (int c0 = 0; c0 < d::NV; c0 += LPS)
+        if (c0 + g.sl < d::NV) w.v[c0 + g.sl] = w.vf[c0 + g.sl];
+    g.sync();
+}
+
+// Projected Gauss-Seidel sweeps (normal row, then the tangent pair with the
+// friction disk |lambda_t| <= mu lambda_n) over nc contacts.  Lane c owns
+// contact c and keeps its residuals rho = b + G lambda + R lambda - v* up to
+// date: every lane projects its own contact, the q-th one's change is broadcast
+// and each lane adds its three rows' share.  NC > 0: at most NC contacts, the
+// lane's Delassus blocks in registers for all sweeps; NC = 0: any number,
+// blocks from shared memory.
 template <int NA, int NC, int LPS>
-__device__ __forceinline__ void pgs_small(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g) {
-    constexpr int NR = 3 * NC;
-    float G[NR][NR], bb[NR], R[NR], iA[NR], vs[NR], lam[NR];
+__device__ __forceinline__ void pgs_sweeps(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g, int nc) {
+    const int c = g.sl < nc ? g.sl : nc - 1;  // lanes past the contacts follow the last one
+    float rho[3], iA[3], lam[3], Gd[2];       // Gd: the own block's normal column
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-#pragma unroll
-        for (int q = 0; q < NR; ++q) G[r][q] = w.ph.con.G[r * NR + q];
-        const float4 c4 = w.ph.con.rc4[r];
-        bb[r] = c4.x;
-        R[r] = c4.y;
-        iA[r] = c4.z;
-        vs[r] = c4.w;
-        lam[r] = 0.0f;
+    for (int k = 0; k < 3; ++k) {
+        rho[k] = w.ph.con.rho[3 * c + k];
+        iA[k] = w.ph.con.iA[3 * c + k];
+        lam[k] = 0.0f;
+        if (k) Gd[k - 1] = w.ph.con.G[(9 * c + 3 * k) * MAXC + c];
     }
-    for (int sw = 0; sw < M.sweeps; ++sw) {
+    const float mu = M.mu;
+    auto contact = [&](int q, const float (&Gq)[9]) {
+        const float ln = fmaxf(__fmaf_rn(-rho[0], iA[0], lam[0]), 0.0f), dn = ln - lam[0];
+        float l1 = __fmaf_rn(-__fmaf_rn(Gd[0], dn, rho[1]), iA[1], lam[1]);
+        float l2 = __fmaf_rn(-__fmaf_rn(Gd[1], dn, rho[2]), iA[2], lam[2]);
+        const float n2 = __fmaf_rn(l1, l1, __fmul_rn(l2, l2)), lim = mu * ln;
+        const float sc = n2 > lim * lim ? lim * rsqrtf(n2) : 1.0f;
+        l1 *= sc;
+        l2 *= sc;
+        const float e0 = g.shfl(dn, q), e1 = g.shfl(l1 - lam[1], q), e2 = g.shfl(l2 - lam[2], q);
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            const int rn = 3 * c;
-            float res = bb[rn] + R[rn] * lam[rn] - vs[rn];
+        for (int k = 0; k < 3; ++k)
+            rho[k] = __fmaf_rn(Gq[3 * k + 2], e2, __fmaf_rn(Gq[3 * k + 1], e1, __fmaf_rn(Gq[3 * k], e0, rho[k])));
+        const bool own = c == q;
+        lam[0] = own ? ln : lam[0];
+        lam[1] = own ? l1 : lam[1];
+        lam[2] = own ? l2 : lam[2];
+    };
+    if constexpr (NC > 0) {
+        float Gq[NC][9];
 #pragma unroll
-            for (int q = 0; q < NR; ++q) res += G[rn][q] * lam[q];
-            const float ln = fmaxf(lam[rn] - res * iA[rn], 0.0f);
-            lam[rn] = ln;
-            float r1 = bb[rn + 1] + R[rn + 1] * lam[rn + 1];
-            float r2 = bb[rn + 2] + R[rn + 2] * lam[rn + 2];
+        for (int q = 0; q < NC; ++q)
 #pragma unroll
-            for (int q = 0; q < NR; ++q) {
-                r1 += G[rn + 1][q] * lam[q];
-                r2 += G[rn + 2][q] * lam[q];
-            }
-            float l1 = lam[rn + 1] - r1 * iA[rn + 1];
-            float l2 = lam[rn + 2] - r2 * iA[rn + 2];
-            const float n2 = l1 * l1 + l2 * l2, lim = M.mu * ln;
-            if (n2 > lim * lim) {
-                const float sc = lim * rsqrtf(n2);
-                l1 *= sc;
-                l2 *= sc;
-            }
-            lam[rn + 1] = l1;
-            lam[rn + 2] = l2;
+            for (int k = 0; k < 9; ++k) Gq[q][k] = q < nc ? w.ph.con.G[(9 * q + k) * MAXC + c] : 0.0f;
+        for (int sw = 0; sw < M.sweeps; ++sw) {
+#pragma unroll
+            for (int q = 0; q < NC; ++q)
+                if (q < nc) contact(q, Gq[q]);
         }
-    }
-    static_assert(NR <= LPS, "one lane per row");
+    } else {
+        for (int sw = 0; sw < M.sweeps; ++sw)
+            for (int q = 0; q < nc; ++q) {
+                float Gq[9];
 #pragma unroll
-    for (int r = 0; r < NR; ++r)
-        if (g.sl == r) w.ph.con.lam[r] = lam[r];
+                for (int k = 0; k < 9; ++k) Gq[k] = w.ph.con.G[(9 * q + k) * MAXC + c];
+                contact(q, Gq);
+            }
+    }
+    if (g.sl < nc) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) w.ph.con.lam[3 * c + k] = lam[k];
+    }
 }
 
 // Soft contact by projected Gauss-Seidel in contact space.  With the
@@ -1290,23 +1415,34 @@ __device__ __forceinline__ void pgs_small(const DevModel& M, WarpWS<NA>& w, cons
 // G = Y Y^T and the unconstrained row velocities are b = Y z_f, z_f = L^T
 // v_f; after the sweeps v = L^-T (z_f + Y^T lambda).  This is the same
 // iteration as updating v row by row (J_r v = b_r + (G lambda)_r).
+// Bound by latency: one warp's chain from the rows through the sweeps
+// (pgs_sweeps).  Cycles of one general contact solve on the planar arms (2.3
+// contacts, 3 sweeps, one warp per scheduler): 6,360 with a reduction of
+// G lambda per residual (five-round butterflies), the rows' branches on the
+// bodies and a Delassus entry per lane; 5,000 with residuals kept per contact
+// and rows against broadcast rows; the planar rollout of 777 samples x 20 steps
+// 150 -> 98 us with the rows' selects, the blocks in registers up to three
+// contacts and the near tests of ball_pass.
 template <int NA, int LPS>
-__device__ __forceinline__ void contacts(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g, int nc, int tb) {
+__device__ __forceinline__ void contacts(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g, const Contacts& con) {
     using d = Dims<NA>;
+    const int nc = con.ncon, tb = con.tb;
     constexpr int SEG = Lanes<LPS>::SEG;
     if (nc == 0) {
-#pragma unroll
-        for (int c0 = 0; c0 < d::NV; c0 += LPS)
-            if (c0 + g.sl < d::NV) w.v[c0 + g.sl] = w.vf[c0 + g.sl];
-        g.sync();
+        free_velocity<NA>(w, g);
         return;
     }
     const float ismb = rsqrtf(M.mb), isIb = rsqrtf(M.Ib);
     // tb: the blocks any contact touches (warp-uniform, from the narrow
     // phase).  Untouched blocks keep v = v_f and skip the z-space work.
-    if (tb == 4 && nc <= 2) {  // ball against static geometry only
-        if (nc == 1) contacts_ball<NA, 1>(M, w, g);
-        else contacts_ball<NA, 2>(M, w, g);
+    if (tb == 4 && nc == 1) {  // ball against static geometry only
+        contacts_ball<NA, 1>(M, w, g, con.floor);
+        return;
+    }
+    store_floor<NA>(M, w, g, con.floor);
+    g.sync();
+    if (tb == 4 && nc == 2) {
+        contacts_ball<NA, 2>(M, w, g, con.floor);
         return;
     }
     // z_f = L^T v_f (one lane per arm coordinate; the ball's lane the ball)
@@ -1331,60 +1467,46 @@ __device__ __forceinline__ void contacts(const DevModel& M, WarpWS<NA>& w, const
     // rows: Jacobian of the touched bodies (in registers), half-solved by
     // the factor, one store per row
     const int nr = 3 * nc;
+    constexpr int NV4 = (d::NV + 3) / 4;
     for (int r = g.sl; r < nr; r += LPS) {
-        const int c = r / 3, k = r - 3 * (r / 3);
+        const int c = r / 3, k = r - 3 * c;
         float e[3];
         contact_frame_row<NA>(w.cn[c], k, e);
         const float* p = w.cp[c];
+        // Jacobian on every block by selects on the bodies (no branches: the
+        // rows of a step have different ones): + on body A, - on body B
+        const int bA = w.cA[c], bB = w.cB[c];
         float ya[2][NA], yb[6];
+        {
+            const float sb = bA == d::B ? 1.0f : (bB == d::B ? -1.0f : 0.0f);
+            const float* bc = &w.q[d::B];
+            const float dd[3] = {p[0] - bc[0], p[1] - bc[1], p[2] - bc[2]};
+            float de[3];
+            cross3(dd, e, de);
 #pragma unroll
-        for (int q = 0; q < NA; ++q) ya[0][q] = ya[1][q] = 0.0f;
-#pragma unroll
-        for (int q = 0; q < 6; ++q) yb[q] = 0.0f;
-        int msk = 0;
-#pragma unroll
-        for (int side = 0; side < 2; ++side) {
-            const int body = side == 0 ? w.cA[c] : w.cB[c];
-            const float sgn = side == 0 ? 1.0f : -1.0f;
-            if (body == d::B) {
-                const float* bc = &w.q[d::B];
-                float dd[3] = {p[0] - bc[0], p[1] - bc[1], p[2] - bc[2]};
-                float de[3];
-                cross3(dd, e, de);
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    yb[q] += sgn * e[q];
-                    yb[3 + q] += sgn * de[q];
-                }
-                msk |= 4;
-            } else if (body >= 0) {
-                const int ab = body >= NA ? 1 : 0;
-                const int ib = body - ab * NA;
-                float col[NA];
-#pragma unroll
-                for (int q = 0; q < NA; ++q) {
-                    col[q] = 0.0f;
-                    if (q <= ib) {
-                        const int lq = ab * NA + q;
-                        float dd[3] = {p[0] - w.o[lq][0], p[1] - w.o[lq][1], p[2] - w.o[lq][2]};
-                        float cz[3];
-                        cross3(w.z[lq], dd, cz);
-                        col[q] = sgn * dot3(e, cz);
-                    }
-                }
-                if (ab == 0) {
-#pragma unroll
-                    for (int q = 0; q < NA; ++q) ya[0][q] += col[q];
-                } else {
-#pragma unroll
-                    for (int q = 0; q < NA; ++q) ya[1][q] += col[q];
-                }
-                msk |= 1 << ab;
+            for (int q = 0; q < 3; ++q) {
+                yb[q] = sb * e[q];
+                yb[3 + q] = sb * de[q];
             }
         }
 #pragma unroll
         for (int ab = 0; ab < 2; ++ab) {
-            if (msk & (1 << ab)) {
+            // joints q <= reach of this arm move the contact (-1: none)
+            const int iA = bA - ab * NA, iB = bB - ab * NA;
+            const bool onA = iA >= 0 && iA < NA, onB = bB >= 0 && iB >= 0 && iB < NA;
+            const int reach = onA ? iA : (onB ? iB : -1);
+            const float sgn = onA ? 1.0f : -1.0f;
+            const float se[3] = {sgn * e[0], sgn * e[1], sgn * e[2]};
+#pragma unroll
+            for (int q = 0; q < NA; ++q) {
+                const int lq = ab * NA + q;
+                const float dd[3] = {p[0] - w.o[lq][0], p[1] - w.o[lq][1], p[2] - w.o[lq][2]};
+                float cz[3];
+                cross3(w.z[lq], dd, cz);
+                const float v = dot3(se, cz);
+                ya[ab][q] = q <= reach ? v : 0.0f;
+            }
+            if ((tb >> ab) & 1) {  // half-solve by the touched arm's factor
 #pragma unroll
                 for (int ii = 0; ii < NA; ++ii) {
                     float sv = ya[ab][ii];
@@ -1394,169 +1516,61 @@ __device__ __forceinline__ void contacts(const DevModel& M, WarpWS<NA>& w, const
                 }
             }
         }
-        float* y = w.ph.con.Y[r];
+        float y[4 * NV4];  // zeros past the last coordinate
 #pragma unroll
-        for (int q = 0; q < NA; ++q) {
-            y[q] = ya[0][q];
-            y[NA + q] = ya[1][q];
-        }
+        for (int q = 0; q < 4 * NV4; ++q)
+            y[q] = q < NA ? ya[0][q < NA ? q : 0]
+                          : q < 2 * NA ? ya[1][q >= NA && q < 2 * NA ? q - NA : 0]
+                                       : q < d::NV ? yb[q >= d::B && q < d::NV ? q - d::B : 0] * (q < d::B + 3 ? ismb : isIb) : 0.0f;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            y[d::B + q] = yb[q] * ismb;
-            y[d::B + 3 + q] = yb[3 + q] * isIb;
-        }
-        w.ph.con.tmask[r] = msk;
-        w.ph.con.rc4[r].w = (k == 0) ? (M.erp / M.dt) * w.cdep[c] : 0.0f;
-        w.ph.con.lam[r] = 0.0f;
+        for (int q = 0; q < NV4; ++q)
+            w.ph.con.Y[r][q] = make_float4(y[4 * q], y[4 * q + 1], y[4 * q + 2], y[4 * q + 3]);
     }
     g.sync();
-    // Delassus block G = Y Y^T (nr x nr) and b = Y z_f, over the blocks rows
-    // share
-    const float regc = (1.0f - M.imp) / M.imp;
-    const int npk = nr * (nr + 1) / 2;
-    for (int t = g.sl; t < npk + nr; t += LPS) {
-        if (t < npk) {
-            // decode (r, s), r <= s, from the upper-triangle index
-            int r = 0, rem = t;
-            while (rem >= nr - r) {
-                rem -= nr - r;
-                ++r;
-            }
-            const int sc = r + rem;
-            const int m = w.ph.con.tmask[r] & w.ph.con.tmask[sc];
-            const float* yr = w.ph.con.Y[r];
-            const float* ys = w.ph.con.Y[sc];
-            float g = 0.0f;
-            if (m & 1) {
+    // Delassus rows G = Y Y^T and b = Y z_f: lane r keeps its row in registers
+    // and reads the others as broadcasts (four partial sums each)
+    const float regc = M.regc;
+    for (int r = g.sl; r < nr; r += LPS) {
+        const int c = r / 3, k = r - 3 * c;
+        float4 yr[NV4];
 #pragma unroll
-                for (int q = 0; q < NA; ++q) g += yr[q] * ys[q];
-            }
-            if (m & 2) {
+        for (int q = 0; q < NV4; ++q) yr[q] = w.ph.con.Y[r][q];
+        float gd = 0.0f;
+        for (int q = 0; q < nc; ++q) {
 #pragma unroll
-                for (int q = NA; q < 2 * NA; ++q) g += yr[q] * ys[q];
-            }
-            if (m & 4) {
+            for (int m = 0; m < 3; ++m) {
+                float p4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-                for (int q = d::B; q < d::NV; ++q) g += yr[q] * ys[q];
+                for (int t = 0; t < NV4; ++t) {
+                    const float4 o = w.ph.con.Y[3 * q + m][t];
+                    p4[0] = __fmaf_rn(yr[t].x, o.x, p4[0]);
+                    p4[1] = __fmaf_rn(yr[t].y, o.y, p4[1]);
+                    p4[2] = __fmaf_rn(yr[t].z, o.z, p4[2]);
+                    p4[3] = __fmaf_rn(yr[t].w, o.w, p4[3]);
+                }
+                float gv = (p4[0] + p4[1]) + (p4[2] + p4[3]);
+                const bool dia = 3 * q + m == r;
+                gv = dia ? __fmaf_rn(regc, gv, gv) : gv;  // A + R, R = regc A
+                gd = dia ? gv : gd;
+                w.ph.con.G[(9 * q + 3 * k + m) * MAXC + c] = gv;
             }
-            w.ph.con.G[r * nr + sc] = g;
-            w.ph.con.G[sc * nr + r] = g;
-            if (sc == r) {
-                const float R = regc * g;
-                w.ph.con.rc4[r].y = R;
-                w.ph.con.rc4[r].z = 1.0f / (g + R);
-            }
-        } else {
-            const int r = t - npk;
-            const int m = w.ph.con.tmask[r];
-            const float* yr = w.ph.con.Y[r];
-            float bb = 0.0f;
-            if (m & 1) {
-#pragma unroll
-                for (int q = 0; q < NA; ++q) bb += yr[q] * w.zz[q];
-            }
-            if (m & 2) {
-#pragma unroll
-                for (int q = NA; q < 2 * NA; ++q) bb += yr[q] * w.zz[q];
-            }
-            if (m & 4) {
-#pragma unroll
-                for (int q = d::B; q < d::NV; ++q) bb += yr[q] * w.zz[q];
-            }
-            w.ph.con.rc4[r].x = bb;
         }
+        w.ph.con.iA[r] = 1.0f / gd;
+        float b4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int q = 0; q < d::NV; ++q) {
+            const int blk = q < NA ? 1 : (q < 2 * NA ? 2 : 4);
+            const float yq = (q & 3) == 0 ? yr[q / 4].x : (q & 3) == 1 ? yr[q / 4].y : (q & 3) == 2 ? yr[q / 4].z : yr[q / 4].w;
+            if (tb & blk) b4[q & 3] = __fmaf_rn(yq, w.zz[q], b4[q & 3]);
+        }
+        const float vs = k == 0 ? M.erp_dt * w.cdep[c] : 0.0f;
+        w.ph.con.rho[r] = ((b4[0] + b4[1]) + (b4[2] + b4[3])) - vs;
     }
     g.sync();
-    // projected Gauss-Seidel sweeps (normal row, then the tangent pair with
-    // the friction disk |lambda_t| <= mu lambda_n).  One or two contacts:
-    // registers.  More: row q's lambda sits on group lane q % LPS as element
-    // q / LPS; the three residuals of a contact are one butterfly reduction
-    // of G_rq lambda_q over the rows (the order of a 32-lane butterfly with
-    // offsets 1, 2, 4, ..., in-lane folds past LPS), and the tangent
-    // residuals take the normal update through G's normal column.
-    if (nc == 1) {
-        pgs_small<NA, 1>(M, w, g);
-    } else if (nc == 2) {
-        pgs_small<NA, 2>(M, w, g);
-    } else {
-        constexpr int RS = 32 / LPS;  // row slots per lane
-        float lamA[RS];
-#pragma unroll
-        for (int t = 0; t < RS; ++t) lamA[t] = 0.0f;
-        int width = 1;
-        while (width < nr && width < 32) width <<= 1;
-        for (int sw = 0; sw < M.sweeps; ++sw) {
-            for (int c = 0; c < nc; ++c) {
-                const int rn = 3 * c;
-                float p0[RS], p1[RS], p2[RS];
-#pragma unroll
-                for (int t = 0; t < RS; ++t) {
-                    const int q = t * LPS + g.sl;
-                    p0[t] = p1[t] = p2[t] = 0.0f;
-                    if (q < nr) {
-                        p0[t] = w.ph.con.G[rn * nr + q] * lamA[t];
-                        p1[t] = w.ph.con.G[(rn + 1) * nr + q] * lamA[t];
-                        p2[t] = w.ph.con.G[(rn + 2) * nr + q] * lamA[t];
-                    }
-                }
-                const float4 cN = w.ph.con.rc4[rn], c1 = w.ph.con.rc4[rn + 1], c2 = w.ph.con.rc4[rn + 2];
-                const float g1n = w.ph.con.G[(rn + 1) * nr + rn];
-                const float g2n = w.ph.con.G[(rn + 2) * nr + rn];
-                for (int off = 1; off < width && off < LPS; off <<= 1) {
-#pragma unroll
-                    for (int t = 0; t < RS; ++t) {
-                        p0[t] += g.xor_(p0[t], off);
-                        p1[t] += g.xor_(p1[t], off);
-                        p2[t] += g.xor_(p2[t], off);
-                    }
-                }
-#pragma unroll
-                for (int st = 1; st < RS; st <<= 1) {
-                    if (st * LPS >= width) break;
-#pragma unroll
-                    for (int t = 0; t + st < RS; t += 2 * st) {
-                        p0[t] += p0[t + st];
-                        p1[t] += p1[t + st];
-                        p2[t] += p2[t + st];
-                    }
-                }
-                // lambda of row r: element r / LPS on group lane r % LPS
-                auto lam_of = [&](int r) {
-                    float v = lamA[0];
-#pragma unroll
-                    for (int t = 1; t < RS; ++t)
-                        if (r / LPS == t) v = lamA[t];
-                    return g.shfl(v, r % LPS);
-                };
-                const float ln0 = lam_of(rn);
-                const float l10 = lam_of(rn + 1);
-                const float l20 = lam_of(rn + 2);
-                const float res = cN.x + p0[0] + cN.y * ln0 - cN.w;
-                const float ln = fmaxf(ln0 - res * cN.z, 0.0f);
-                const float dn = ln - ln0;
-                const float r1 = c1.x + p1[0] + g1n * dn + c1.y * l10;
-                const float r2 = c2.x + p2[0] + g2n * dn + c2.y * l20;
-                float l1 = l10 - r1 * c1.z;
-                float l2 = l20 - r2 * c2.z;
-                const float n2 = l1 * l1 + l2 * l2, lim = M.mu * ln;
-                if (n2 > lim * lim) {
-                    const float sc = lim * rsqrtf(n2);
-                    l1 *= sc;
-                    l2 *= sc;
-                }
-#pragma unroll
-                for (int t = 0; t < RS; ++t) {
-                    const int q = t * LPS + g.sl;
-                    if (q == rn) lamA[t] = ln;
-                    if (q == rn + 1) lamA[t] = l1;
-                    if (q == rn + 2) lamA[t] = l2;
-                }
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < RS; ++t)
-            if (t * LPS + g.sl < nr) w.ph.con.lam[t * LPS + g.sl] = lamA[t];
-    }
+    // projected Gauss-Seidel sweeps
+    if (nc <= 2) pgs_sweeps<NA, 2>(M, w, g, nc);
+    else if (nc == 3) pgs_sweeps<NA, 3>(M, w, g, nc);
+    else pgs_sweeps<NA, 0>(M, w, g, nc);
     g.sync();
     // z = z_f + Y^T lambda, then v = L^-T z on the touched blocks
 #pragma unroll
@@ -1565,9 +1579,13 @@ __device__ __forceinline__ void contacts(const DevModel& M, WarpWS<NA>& w, const
         if (c < d::NV) {
             const int blk = c < NA ? 1 : (c < 2 * NA ? 2 : 4);
             if (tb & blk) {
-                float zv = w.zz[c];
-                for (int r = 0; r < nr; ++r) zv += w.ph.con.Y[r][c] * w.ph.con.lam[r];
-                w.zz[c] = zv;
+                float z3[3] = {w.zz[c], 0.0f, 0.0f};
+                for (int q = 0; q < nc; ++q)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        z3[k] = __fmaf_rn(reinterpret_cast<const float*>(&w.ph.con.Y[3 * q + k][c / 4])[c & 3],
+                                          w.ph.con.lam[3 * q + k], z3[k]);
+                w.zz[c] = z3[0] + (z3[1] + z3[2]);
             } else {
                 w.v[c] = w.vf[c];
             }

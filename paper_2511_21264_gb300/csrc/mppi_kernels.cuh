@@ -134,24 +134,24 @@ __device__ __forceinline__ float rollout_sample(const DevModel& M, WarpWS<NA>& w
         // formed before the collision phase, so that the link frames kept
         // from the kinematics are no longer live across it
         dynamics<NA>(M, w, g, io.err, Rl, cl, 0, false);
-        int ncon, tb;
-        n_exact += collide<NA>(M, w, g, pacc, pbacc, ncon, tb);
+        Contacts con;
+        collide<NA>(M, w, g, pacc, pbacc, con);
         g.sync();
-        n_con += ncon;
+        if (con.nsurv > 0) {
+            n_exact += sl == 0 ? con.nsurv : 0;
+            collide_exact<NA>(M, w, g, pacc, pbacc, con);
+            g.sync();
+        }
+        n_con += con.ncon;
         // one ball contact with static geometry (the lift's common case)
-        const bool lone = tb == 4 && ncon == 1;
+        const bool lone = con.tb == 4 && con.ncon == 1;
         n_lone += lone ? 1u : 0u;
-        if (PLACE == 0) {
+        if (PLACE == 0 && lone) {
             // the arms' solve and the contact solve side by side
-            if (lone) {
-                solve_ball_contacts<NA, 1, 0>(M, w, g, io.err);
-            } else {
-                arm_factor_step<NA, LPS>(M, w, g, io.err, tb);
-                contacts<NA>(M, w, g, ncon, tb);
-            }
+            solve_ball_contact<NA>(M, w, g, io.err, con.floor);
         } else {
-            arm_factor_step<NA, LPS>(M, w, g, io.err, tb);
-            contacts<NA>(M, w, g, ncon, tb);
+            arm_factor_step<NA, LPS>(M, w, g, io.err, con.tb);
+            contacts<NA>(M, w, g, con);
         }
         integrate<NA>(M, w, g);
         if (!TASK && sl < 3) {  // the goal error of ball coordinate sl

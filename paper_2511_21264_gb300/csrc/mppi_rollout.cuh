@@ -23,18 +23,25 @@ namespace mppi {
 // 128 / (samples per warp) bytes apart modulo 128, so that the groups'
 // lane-indexed shared-memory accesses fall in different banks.
 template <int NA, int LPS>
-__host__ __device__ constexpr size_t ws_stride() {
+__host__ __device__ constexpr size_t ws_stride(size_t at_least = 0) {
     size_t s = (sizeof(WarpWS<NA>) + 31) / 32 * 32;
+    if (s < at_least) s = at_least;
     if (LPS == 32) return s;
     const size_t want = 128 / (32 / LPS);
     while (s % 128 != want) s += 32;
     return s;
 }
+// The single controller's stride does not follow a smaller workspace: the
+// samples per CTA that its launches accept stay what they are.
+template <int NA, int LPS>
+__host__ __device__ constexpr size_t ctl_stride() {
+    return ws_stride<NA, LPS>(NA == 7 ? 7328 : 5600);
+}
 
 template <int NA, int LPS>
 size_t rollout_smem(int spc, int unom_floats, bool task) {
     return sizeof(DevModel) + (task ? sizeof(DevTask) : 0) + ((size_t)unom_floats * sizeof(float) + 15) / 16 * 16 +
-           (size_t)spc * ws_stride<NA, LPS>();
+           (size_t)spc * ctl_stride<NA, LPS>();
 }
 
 template <int NA, int LPS, int MODE, bool TASK, int PLACE>
@@ -63,7 +70,7 @@ __global__ void __launch_bounds__(512) rollout_kernel(RolloutArgs args) {
     const Lanes<LPS> g(threadIdx.x & 31);
     const int k = blockIdx.x * spc + gi;
     if (k >= args.n) return;
-    WarpWS<NA>& w = *reinterpret_cast<WarpWS<NA>*>(smem + ws_off + (size_t)gi * ws_stride<NA, LPS>());
+    WarpWS<NA>& w = *reinterpret_cast<WarpWS<NA>*>(smem + ws_off + (size_t)gi * ctl_stride<NA, LPS>());
     SampleIO io{};
     io.x = args.states + (size_t)k * args.state_stride;
     io.k = k;
