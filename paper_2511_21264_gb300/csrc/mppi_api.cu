@@ -262,7 +262,7 @@ struct mppi_ctx {
     int K = 0, H = 0, spc = 4;
     int lps = 32, place = 0;  // lanes per sample, placement of the lone ball contact's solve
     bool spc_auto = true;     // spc is the library's choice for the layout
-    int spc_alt = 0, spc_alt_lps = 0;  // the default shape of another layout (the task suite's)
+    int spc_task = 0, spc_task_lps = 0;  // the ball-task suite's default shape in layout spc_task_lps
     float lambda = 1.0f;
     uint64_t seed = 0;
     float* d_sigma = nullptr;
@@ -410,26 +410,33 @@ int mppi_destroy(mppi_ctx* c) {
 // Samples per rollout CTA when the caller sets none: the shape that puts
 // the K samples on the SMs in the fewest waves with the least load on the
 // busiest SM (occupancy of the sampling rollout kernel of the layout).
-static int default_spc_for(const mppi_ctx* c, int lps) {
-    const int unom = c->H * 2 * c->m->info.na <= 2048 ? c->H * 2 * c->m->info.na : 0;
-    return c->m->info.na == 3 ? choose_spc_na3(lps, c->K, unom) : choose_spc_na7(lps, c->K, unom);
+static int unom_floats(const mppi_ctx* c) { return c->H * 2 * c->m->info.na <= 2048 ? c->H * 2 * c->m->info.na : 0; }
+static int default_spc_for(const mppi_ctx* c, int lps, bool task) {
+    return c->m->info.na == 3 ? choose_spc_na3(lps, c->K, unom_floats(c), task)
+                              : choose_spc_na7(lps, c->K, unom_floats(c), task);
 }
-static int default_spc(const mppi_ctx* c) { return default_spc_for(c, c->lps); }
+static int default_spc(const mppi_ctx* c) { return default_spc_for(c, c->lps, false); }
 
-// Samples per CTA for a launch in layout lps: the handle's shape when lps is
-// its layout, else (the ball-task suite runs on 32 lanes per sample) the
-// default shape for lps, or the handle's shape capped at 512 threads when
-// the caller chose it.
-static int launch_spc(mppi_ctx* c, int lps) {
-    if (lps == c->lps) return c->spc;
+// Layout and samples per CTA of a rollout: the handle's.  The ball-task suite
+// needs a lane per link and its own points in shared memory: it runs on 32
+// lanes where the handle has 8, and with its own default shape; a shape that the
+// caller chose is kept, on 32 lanes (at most 512 threads) where it does not fit.
+static int rollout_shape(mppi_ctx* c, RolloutArgs* a) {
+    a->lps = c->lps;
+    a->place = c->place;
+    if (!a->task) return c->spc;
+    a->place = 0;
+    if (c->lps == 8) a->lps = 32;
     if (c->spc_auto) {
-        if (c->spc_alt_lps != lps) {
-            c->spc_alt = default_spc_for(c, lps);
-            c->spc_alt_lps = lps;
+        if (c->spc_task_lps != a->lps) {
+            c->spc_task = default_spc_for(c, a->lps, true);
+            c->spc_task_lps = a->lps;
         }
-        return c->spc_alt;
+        return c->spc_task;
     }
-    return std::min(c->spc, 512 / lps);
+    const int n = unom_floats(c);
+    if (a->lps == 16 && !(c->m->info.na == 3 ? task_fits<3>(c->spc, n) : task_fits<7>(c->spc, n))) a->lps = 32;
+    return a->lps == c->lps ? c->spc : std::min(c->spc, 512 / a->lps);
 }
 
 int mppi_create(const mppi_model* m, int K, int H, float lambda, const float* sigma, uint64_t seed, mppi_ctx** out) {
@@ -706,8 +713,6 @@ static RolloutArgs philox_args(mppi_ctx* c, const float* state, const float* u_n
     a.U_store = c->d_U;
     a.Lfac = c->cov_sampling ? c->d_L : nullptr;
     a.task = c->task_on ? c->d_task : nullptr;
-    a.lps = a.task ? 32 : c->lps;  // the ball-task suite runs on 32 lanes per sample
-    a.place = a.task ? 0 : c->place;
     return a;
 }
 
@@ -979,9 +984,10 @@ static int enqueue_step(mppi_ctx* c, const float* state, const float* u_nom, flo
     // dependent CTAs cost more than the overlap saves (lift, K = 1024: 0.146
     // ms per iteration without, 0.168 with), so they are used with wider CTAs
     // only; event records between the kernels would break the overlap anyway.
-    const bool pdl = !prof && launch_spc(c, a.lps) * a.lps > 32;
+    const int spc = rollout_shape(c, &a);
+    const bool pdl = !prof && spc * a.lps > 32;
     a.pdl = pdl;
-    rc = launch_rollout(c->m->info.na, mode, a, launch_spc(c, a.lps), s);
+    rc = launch_rollout(c->m->info.na, mode, a, spc, s);
     if (rc != MPPI_OK) return rc;
     if (prof) cudaEventRecord(ev[2], s);
     if (elite_mode(c)) {
@@ -1102,8 +1108,8 @@ int rollout_batch(mppi_ctx* c, int n, const float* states, const float* U, float
     a.states_out = states_out;
     a.err = c->d_err;
     a.task = c->task_on ? c->d_task : nullptr;
-    a.lps = a.task ? 32 : c->lps;
-    return launch_rollout(c->m->info.na, 0, a, launch_spc(c, a.lps), (cudaStream_t)stream);
+    const int spc = rollout_shape(c, &a);
+    return launch_rollout(c->m->info.na, 0, a, spc, (cudaStream_t)stream);
 }
 
 int sim_step(mppi_ctx* c, int n, float* states, const float* U1, void* stream) {
@@ -1118,8 +1124,8 @@ int sim_step(mppi_ctx* c, int n, float* states, const float* U1, void* stream) {
     a.costs = c->d_costs;
     a.states_out = states;  // each lane group reads its state before writing it back
     a.err = c->d_err;
-    a.lps = c->lps;
-    return launch_rollout(c->m->info.na, 0, a, launch_spc(c, a.lps), (cudaStream_t)stream);
+    const int spc = rollout_shape(c, &a);
+    return launch_rollout(c->m->info.na, 0, a, spc, (cudaStream_t)stream);
 }
 
 int mppi_debug_noise(mppi_ctx* c, uint64_t iteration, float* eps, void* stream) {

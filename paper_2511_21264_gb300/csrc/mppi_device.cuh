@@ -179,6 +179,11 @@ struct __align__(16) WarpWS {
             CArr<float, MAXR> iA;        // 1 / (A + R)
             CArr<float, MAXR> lam;
         } con;
+        struct {  // ball-task suite: the pairs whose distances are needed
+            CArr<float, 2 * MAXL + 2> motion;                             // of each link's ends since the last state
+            CArr<short, 2 * MAXL * MAXB + 2 * MAXL + MAXL * MAXL + 1> pair;  // in pair order; 0x4000: dist holds the previous one
+            CArr<float, 2 * MAXL * MAXB + 2 * MAXL + MAXL * MAXL> dist;
+        } task;
     } ph;
 };
 

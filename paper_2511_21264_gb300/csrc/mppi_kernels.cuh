@@ -37,7 +37,7 @@ __device__ __forceinline__ void stage_model(unsigned char* smem, const DevModel*
 }
 
 // H simulator steps of one sample with its stage costs (TASK: the ball-task
-// cost suite instead, 32 lanes per sample only); the group's state stays in
+// cost suite instead, on 32 or 16 lanes); the group's state stays in
 // shared memory throughout.  PLACE selects where the lone ball contact's
 // solve runs: 0 fused with the arms' factorisation (every lane runs both
 // chains), 1 after it (the factor on one lane per arm, then the sweeps);
@@ -46,7 +46,7 @@ template <int NA, int LPS, int MODE, bool TASK = false, int PLACE = 0>
 __device__ __forceinline__ float rollout_sample(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g,
                                                 const SampleIO& io) {
     using d = Dims<NA>;
-    static_assert(!TASK || LPS == 32, "the ball-task cost suite runs on 32 lanes per sample");
+    static_assert(!TASK || LPS >= 16, "the ball-task cost suite takes one lane per link");
     static_assert(d::NU <= LPS, "one lane per control");
     constexpr int PS = 32 / LPS;  // pair slots per lane
     constexpr int DS = LPS / 4;   // steps of normals per Philox draw (one block of 4 per lane)
@@ -68,13 +68,11 @@ __device__ __forceinline__ float rollout_sample(const DevModel& M, WarpWS<NA>& w
     for (int t = 0; t < PS; ++t) pacc[t] = pbacc[t] = 0.0f;
     float gacc = 0.0f;  // squared goal error of this lane's ball coordinate over the horizon
     float kacc = 0.0f;  // squared grasp error (p_L + p_R - 2 p_ball) of this lane's coordinate
-    TaskAcc<NA> tacc;
+    TaskAcc<NA, LPS> tacc;
     if constexpr (TASK) {
 #pragma unroll
-        for (int s = 0; s < TaskDims<NA>::CB; ++s) tacc.prevb[s] = 0.0f;
-#pragma unroll
-        for (int s = 0; s < TaskDims<NA>::CC; ++s) tacc.prevc[s] = 0.0f;
-        tacc.c = tacc.th = tacc.yz = tacc.v2 = tacc.r = tacc.l = tacc.eo = tacc.ot = 0.0f;
+        for (int t = 0; t < PS; ++t) tacc.c[t] = 0.0f;
+        tacc.th = tacc.yz = tacc.v2 = tacc.r = tacc.l = tacc.eo = tacc.ot = 0.0f;
     }
     float upre = 0.0f;  // explicit controls: the next step's value
     if (MODE == 0 && sl < d::NU) upre = ld_checked(io.U, sl, io.u_ext);
@@ -126,7 +124,7 @@ __device__ __forceinline__ float rollout_sample(const DevModel& M, WarpWS<NA>& w
         forward_kinematics<NA>(M, w, g, Rl, cl);
         g.sync();
         if constexpr (TASK) {
-            task_state<NA>(M, *io.task, w, sl, Rl, h == 0, tacc);
+            task_state<NA, LPS>(M, *io.task, w, g, Rl, h == 0, tacc);
         } else {
             if (h > 0 && sl < 3 && M.w_grasp != 0.0f) kacc += grasp_coord<NA>(w, sl);
         }
@@ -164,8 +162,8 @@ __device__ __forceinline__ float rollout_sample(const DevModel& M, WarpWS<NA>& w
         float Rl[9], cl[3];
         forward_kinematics<NA>(M, w, g, Rl, cl);
         g.sync();
-        task_state<NA>(M, *io.task, w, sl, Rl, false, tacc);
-        cost = task_total<NA>(*io.task, tacc);
+        task_state<NA, LPS>(M, *io.task, w, g, Rl, false, tacc);
+        cost = task_total<NA, LPS>(*io.task, g, tacc);
     } else if (M.w_grasp != 0.0f) {
         float Rl[9], cl[3];
         forward_kinematics<NA>(M, w, g, Rl, cl);

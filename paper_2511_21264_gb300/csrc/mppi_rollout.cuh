@@ -24,8 +24,9 @@ namespace mppi {
 // lane-indexed shared-memory accesses fall in different banks.
 template <int NA, int LPS>
 __host__ __device__ constexpr size_t ws_stride(size_t at_least = 0) {
-    size_t s = (sizeof(WarpWS<NA>) + 31) / 32 * 32;
+    size_t s = sizeof(WarpWS<NA>);
     if (s < at_least) s = at_least;
+    s = (s + 31) / 32 * 32;
     if (LPS == 32) return s;
     const size_t want = 128 / (32 / LPS);
     while (s % 128 != want) s += 32;
@@ -33,15 +34,17 @@ __host__ __device__ constexpr size_t ws_stride(size_t at_least = 0) {
 }
 // The single controller's stride does not follow a smaller workspace: the
 // samples per CTA that its launches accept stay what they are.
-template <int NA, int LPS>
+// The ball-task suite keeps the previous state's points behind the workspace.
+template <int NA, int LPS, bool TASK>
 __host__ __device__ constexpr size_t ctl_stride() {
-    return ws_stride<NA, LPS>(NA == 7 ? 7328 : 5600);
+    constexpr size_t least = NA == 7 ? 7328 : 5600, task = sizeof(WarpWS<NA>) + sizeof(TaskPrev<NA>);
+    return ws_stride<NA, LPS>(TASK && task > least ? task : least);
 }
 
-template <int NA, int LPS>
-size_t rollout_smem(int spc, int unom_floats, bool task) {
-    return sizeof(DevModel) + (task ? sizeof(DevTask) : 0) + ((size_t)unom_floats * sizeof(float) + 15) / 16 * 16 +
-           (size_t)spc * ctl_stride<NA, LPS>();
+template <int NA, int LPS, bool TASK>
+size_t rollout_smem(int spc, int unom_floats) {
+    return sizeof(DevModel) + (TASK ? sizeof(DevTask) : 0) + ((size_t)unom_floats * sizeof(float) + 15) / 16 * 16 +
+           (size_t)spc * ctl_stride<NA, LPS, TASK>();
 }
 
 template <int NA, int LPS, int MODE, bool TASK, int PLACE>
@@ -70,7 +73,7 @@ __global__ void __launch_bounds__(512) rollout_kernel(RolloutArgs args) {
     const Lanes<LPS> g(threadIdx.x & 31);
     const int k = blockIdx.x * spc + gi;
     if (k >= args.n) return;
-    WarpWS<NA>& w = *reinterpret_cast<WarpWS<NA>*>(smem + ws_off + (size_t)gi * ctl_stride<NA, LPS>());
+    WarpWS<NA>& w = *reinterpret_cast<WarpWS<NA>*>(smem + ws_off + (size_t)gi * ctl_stride<NA, LPS, TASK>());
     SampleIO io{};
     io.x = args.states + (size_t)k * args.state_stride;
     io.k = k;
@@ -118,7 +121,7 @@ inline int cuda_fail(cudaError_t e) {
 template <int NA, int LPS, int MODE, bool TASK, int PLACE>
 int launch_t(const RolloutArgs& a, int spc, cudaStream_t s) {
     const int unom = (MODE >= 1 && a.stage_unom) ? a.H * Dims<NA>::NU : 0;
-    const size_t sm = rollout_smem<NA, LPS>(spc, unom, TASK);
+    const size_t sm = rollout_smem<NA, LPS, TASK>(spc, unom);
     auto fn = rollout_kernel<NA, LPS, MODE, TASK, PLACE>;
     int dev = 0, max_sm = 0;
     cudaError_t q = cudaGetDevice(&dev);
@@ -151,11 +154,17 @@ int launch_lps(int mode, const RolloutArgs& a, int spc, cudaStream_t s) {
     return a.place ? launch_t<NA, LPS, 1, false, 1>(a, spc, s) : launch_t<NA, LPS, 1, false, 0>(a, spc, s);
 }
 
+template <int NA, int LPS>
+int launch_task(int mode, const RolloutArgs& a, int spc, cudaStream_t s) {
+    if (mode == 0) return launch_t<NA, LPS, 0, true, 0>(a, spc, s);
+    return a.Lfac ? launch_t<NA, LPS, 2, true, 0>(a, spc, s) : launch_t<NA, LPS, 1, true, 0>(a, spc, s);
+}
+
 }  // namespace rollout_launch
 
 // Launch for one arm size.  a.lps (0 = 32) and a.place select the layout;
-// spc is rounded up to whole warps.  The ball-task suite runs on 32 lanes
-// per sample with the fused placement only.  A shape whose workspaces do not
+// spc is rounded up to whole warps.  The ball-task suite runs on 32 or 16
+// lanes per sample with the fused placement only.  A shape whose workspaces do not
 // fit one CTA's shared memory is refused with MPPI_ERR_INVALID_ARG.
 template <int NA>
 int dispatch_rollout(int mode, const RolloutArgs& a, int spc, cudaStream_t s) {
@@ -167,9 +176,8 @@ int dispatch_rollout(int mode, const RolloutArgs& a, int spc, cudaStream_t s) {
     spc = (spc + spw - 1) / spw * spw;
     if (spc * lps > 512) return MPPI_ERR_INVALID_ARG;
     if (a.task) {
-        if (lps != 32 || a.place != 0) return MPPI_ERR_UNSUPPORTED;
-        if (mode == 0) return launch_t<NA, 32, 0, true, 0>(a, spc, s);
-        return a.Lfac ? launch_t<NA, 32, 2, true, 0>(a, spc, s) : launch_t<NA, 32, 1, true, 0>(a, spc, s);
+        if (lps == 8 || a.place != 0) return MPPI_ERR_UNSUPPORTED;
+        return lps == 32 ? launch_task<NA, 32>(mode, a, spc, s) : launch_task<NA, 16>(mode, a, spc, s);
     }
     if (lps == 32) return launch_lps<NA, 32>(mode, a, spc, s);
     if (lps == 16) return launch_lps<NA, 16>(mode, a, spc, s);
@@ -184,8 +192,18 @@ int dispatch_rollout(int mode, const RolloutArgs& a, int spc, cudaStream_t s) {
 // the busiest SM, then the larger CTA (fewer model copies to stage; on
 // GB300 a 28-sample CTA per SM beat two 14-sample CTAs by 5%); past one wave
 // the most samples resident per SM, then the smaller CTA.
+template <int NA, int LPS, bool TASK>
+bool spc_occupancy(int spc, int unom_floats, int max_sm, int* per_sm) {
+    const auto fn = rollout_kernel<NA, LPS, 1, TASK, 0>;
+    const size_t sm = rollout_smem<NA, LPS, TASK>(spc, unom_floats);
+    *per_sm = 0;
+    return sm <= (size_t)max_sm &&
+           cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess &&
+           cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, fn, spc * LPS, sm) == cudaSuccess && *per_sm > 0;
+}
+
 template <int NA>
-int choose_spc(int lps, int K, int unom_floats) {
+int choose_spc(int lps, int K, int unom_floats, bool task) {
     int dev = 0, nsm = 0, max_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -195,38 +213,18 @@ int choose_spc(int lps, int K, int unom_floats) {
     long best_w = 1L << 40, best_key = 1L << 40;
     int best = spw;
     for (int spc = spw; spc * lps <= 512; spc += spw) {
-        size_t sm = 0;
         int per_sm = 0;
-        cudaError_t e = cudaSuccess;
+        bool ok = false;
         if (lps == 32) {
-            sm = rollout_smem<NA, 32>(spc, unom_floats, false);
-            if (sm <= (size_t)max_sm) {
-                e = cudaFuncSetAttribute(rollout_kernel<NA, 32, 1, false, 0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-                if (e == cudaSuccess)
-                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rollout_kernel<NA, 32, 1, false, 0>,
-                                                                      spc * 32, sm);
-            }
+            ok = task ? spc_occupancy<NA, 32, true>(spc, unom_floats, max_sm, &per_sm)
+                      : spc_occupancy<NA, 32, false>(spc, unom_floats, max_sm, &per_sm);
         } else if (lps == 16) {
-            sm = rollout_smem<NA, 16>(spc, unom_floats, false);
-            if (sm <= (size_t)max_sm) {
-                e = cudaFuncSetAttribute(rollout_kernel<NA, 16, 1, false, 0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-                if (e == cudaSuccess)
-                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rollout_kernel<NA, 16, 1, false, 0>,
-                                                                      spc * 16, sm);
-            }
+            ok = task ? spc_occupancy<NA, 16, true>(spc, unom_floats, max_sm, &per_sm)
+                      : spc_occupancy<NA, 16, false>(spc, unom_floats, max_sm, &per_sm);
         } else if constexpr (Lanes<8>::SEG > NA) {
-            sm = rollout_smem<NA, 8>(spc, unom_floats, false);
-            if (sm <= (size_t)max_sm) {
-                e = cudaFuncSetAttribute(rollout_kernel<NA, 8, 1, false, 0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-                if (e == cudaSuccess)
-                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rollout_kernel<NA, 8, 1, false, 0>,
-                                                                      spc * 8, sm);
-            }
+            ok = !task && spc_occupancy<NA, 8, false>(spc, unom_floats, max_sm, &per_sm);
         }
-        if (e != cudaSuccess || per_sm <= 0) continue;
+        if (!ok) continue;
         const long blocks = (K + spc - 1) / spc;
         const long cap = (long)per_sm * nsm;
         const long waves = (blocks + cap - 1) / cap;
@@ -243,6 +241,15 @@ int choose_spc(int lps, int K, int unom_floats) {
     return best;
 }
 
+// Whether a launch of spc samples per CTA fits one CTA's shared memory.
+template <int NA>
+bool task_fits(int spc, int unom_floats) {
+    int dev = 0, max_sm = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&max_sm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+           rollout_smem<NA, 16, true>((spc + 1) / 2 * 2, unom_floats) <= (size_t)max_sm;
+}
+
 // Default layout for K samples: 16 lanes per sample once 32-lane groups
 // cannot hold all K samples in one wave (their registers allow 16 warps per
 // SM), else 32 (the shorter per-step chain of one sample per warp).
@@ -256,7 +263,7 @@ inline int default_lps(int K) {
 
 int launch_rollout_na7(int mode, const RolloutArgs& a, int spc, cudaStream_t s);
 int launch_rollout_na3(int mode, const RolloutArgs& a, int spc, cudaStream_t s);
-int choose_spc_na7(int lps, int K, int unom_floats);
-int choose_spc_na3(int lps, int K, int unom_floats);
+int choose_spc_na7(int lps, int K, int unom_floats, bool task);
+int choose_spc_na3(int lps, int K, int unom_floats, bool task);
 
 }  // namespace mppi

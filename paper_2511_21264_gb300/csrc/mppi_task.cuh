@@ -1,8 +1,7 @@
 // The paper's ball-task cost suite (Sec. IV-B) evaluated inside the rollout:
-// per state, the signed distances of the collision pairs (one lane per
-// pair), the end effectors' positions, orientations and velocities, and the
-// per-state terms; the barrier keeps each pair's previous distance in the
-// lane's registers.
+// per state, the signed distances of the collision pairs that can enter the
+// barrier or the penetration count, the end effectors' positions, orientations
+// and velocities, and the per-state terms.
 #pragma once
 #include "mppi_device.cuh"
 
@@ -20,20 +19,30 @@ struct __align__(16) DevTask {
 };
 
 // pairs: links x boxes (link-major) in the first lane passes, then links x
-// ball (pick) and left x right links, so that every pass evaluates one kind
-template <int NA>
+// ball (pick) and left x right links, so that every pass holds one kind
+template <int NA, int LPS>
 struct TaskDims {
-    static constexpr int CB = (2 * NA * MAXB + 31) / 32;  // capsule-box passes at most
-    static constexpr int CC = (2 * NA + NA * NA + 31) / 32;
+    static constexpr int CB = (2 * NA * MAXB + LPS - 1) / LPS;  // capsule-box passes at most
+    static constexpr int CC = (2 * NA + NA * NA + LPS - 1) / LPS;
+    static_assert(CB + CC <= 32, "one bit per pass");
 };
 
-template <int NA>
+template <int NA, int LPS>
 struct TaskAcc {
-    float prevb[TaskDims<NA>::CB];  // each pass's pair distance at the previous state (this lane)
-    float prevc[TaskDims<NA>::CC];
-    float c;                        // barrier + penetration count (this lane)
+    // this lane's pairs, one per pass: a lower bound of the pair's distance at
+    // the previous state, the distance itself where the bit of exact is set
+    float lb[TaskDims<NA, LPS>::CB + TaskDims<NA, LPS>::CC];
+    unsigned exact;
+    float c[32 / LPS];              // barrier + penetration count, per slot of the pair list
     float r;                        // orientation error (the end-effector lanes)
     float th, yz, v2, l, eo, ot;    // per-state terms (lane 0)
+};
+
+// The previous state's capsule ends and ball, behind the sample's workspace.
+template <int NA>
+struct __align__(16) TaskPrev {
+    CArr<CArr<float, 6>, 2 * NA> a;
+    CArr<float, 4> ball;
 };
 
 // Minimum over t in [0,1] of the box SDF f(t) at a0 + t dd, for any segment
@@ -248,50 +257,174 @@ __device__ __forceinline__ float quat_angle(const float* q, const float* qs) {
 // Task terms of the state whose kinematics forward_kinematics just wrote
 // (w.a0/a1/z/o, Rl on the lane of each link).  first: the present state
 // x_0, which only seeds the barrier's previous distances.
-template <int NA>
-__device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, WarpWS<NA>& w, int lane,
-                                           const float (&Rl)[9], bool first, TaskAcc<NA>& acc) {
+//
+// A pair adds to the cost only when its distance falls below (1 - gamma) of the
+// previous one (gamma < 1, so a penetrating pair always does).  A distance
+// changes by at most the motion of the pair's ends, so a pair whose lower bound
+// at the previous state is above motion / gamma adds nothing: its bound drops by
+// the motion and no distance is formed.  The others (near or fast ones, a few of
+// up to 287) go to a list in pair order, spread over the group's lanes, each
+// with its distance now and, unless that is known from the previous state, the
+// one before.  The margins (1e-5 of the motion, 2e-5 m) are far above the
+// rounding of the distances, so the terms are those of testing every pair.
+// MEASURED_TASK
+template <int NA, int LPS>
+__device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, WarpWS<NA>& w, const Lanes<LPS>& g,
+                                           const float (&Rl)[9], bool first, TaskAcc<NA, LPS>& acc) {
     using d = Dims<NA>;
-    const int nlb = 2 * NA * M.nb;
-    const int ncb = (nlb + 31) >> 5;  // capsule-box passes
+    using td = TaskDims<NA, LPS>;
+    constexpr int PS = 32 / LPS;
+    TaskPrev<NA>& pv = *reinterpret_cast<TaskPrev<NA>*>(&w + 1);
+    const int nb = M.nb, nlb = 2 * NA * nb;
+    const int ncb = (nlb + LPS - 1) / LPS;  // capsule-box passes
     const int nball = T.phase == 0 ? 2 * NA : 0;
     const int ncc = nball + NA * NA;
     const float keep = 1.0f - T.gamma;
-    // capsule-box passes: one copy of the code, the pass's previous
-    // distance picked out of the register array by selects
+    // ball-link and link-link pair b: the ball is a capsule of zero length
+    auto segment_pair = [&](int b, bool now) {
+        const bool ball = b < nball;
+        const int r = b - nball, i = r / NA, j = r - i * NA;
+        const int la = ball ? b : i, lb = ball ? 0 : NA + j;
+        const float* x0 = now ? &w.a0[la][0] : &pv.a[la][0];
+        const float* x1 = now ? &w.a1[la][0] : &pv.a[la][3];
+        const float* c0 = ball ? (now ? &w.q[d::B] : &pv.ball[0]) : (now ? &w.a0[lb][0] : &pv.a[lb][0]);
+        const float* c1 = ball ? c0 : (now ? &w.a1[lb][0] : &pv.a[lb][3]);
+        return capsule_capsule_distance(x0, x1, M.link[la / NA][la % NA].rcap, c0, c1, ball ? M.rb : M.link[1][j].rcap);
+    };
+    if (first) {
 #pragma unroll 1
-    for (int s = 0; s < ncb; ++s) {
-        const int b = lane + 32 * s;
-        if (b < nlb) {
-            const int l = b / M.nb, bx = b - l * M.nb;
-            const float dist = capsule_box_distance(w.a0[l], w.a1[l], M.link[l / NA][l % NA].rcap, M.box[bx]);
-            float pv = acc.prevb[0];
+        for (int s = 0; s < ncb; ++s) {
+            const int b = g.sl + LPS * s;
+            if (b < nlb) {
+                const int l = b / nb, bx = b - l * nb;
+                acc.lb[s] = capsule_box_distance(w.a0[l], w.a1[l], M.link[l / NA][l % NA].rcap, M.box[bx]);
+            }
+        }
+#pragma unroll 1
+        for (int s = 0; s < td::CC; ++s) {
+            const int b = g.sl + LPS * s;
+            if (b < ncc) acc.lb[td::CB + s] = segment_pair(b, true);
+        }
+        acc.exact = ~0u;
+    } else {
+        auto& sc = w.ph.task;
+        // motion of every link's ends and of the ball since the previous state
+        if (g.sl < 2 * NA) {
+            float m0 = 0.0f, m1 = 0.0f;
 #pragma unroll
-            for (int k = 1; k < TaskDims<NA>::CB; ++k) pv = s == k ? acc.prevb[k] : pv;
-            if (!first) acc.c += fmaxf(-dist + keep * pv, 0.0f) + (dist < 0.0f ? 1.0f : 0.0f);
+            for (int k = 0; k < 3; ++k) {
+                const float e0 = w.a0[g.sl][k] - pv.a[g.sl][k], e1 = w.a1[g.sl][k] - pv.a[g.sl][3 + k];
+                m0 = __fmaf_rn(e0, e0, m0);
+                m1 = __fmaf_rn(e1, e1, m1);
+            }
+            sc.motion[g.sl] = sqrtf(fmaxf(m0, m1));
+        }
+        float mb = 0.0f;
 #pragma unroll
-            for (int k = 0; k < TaskDims<NA>::CB; ++k) acc.prevb[k] = s == k ? dist : acc.prevb[k];
+        for (int k = 0; k < 3; ++k) {
+            const float e = w.q[d::B + k] - pv.ball[k];
+            mb = __fmaf_rn(e, e, mb);
+        }
+        mb = sqrtf(mb);
+        g.sync();
+        int nlist = 0;
+        unsigned trig = 0u;
+        // a pair of pass bit s: screened, or put on the list with its bound
+        auto screen = [&](int s, int b, bool in, float motion) {
+            const float lbv = acc.lb[s], need = __fmaf_rn(motion, 1.00001f, 2e-5f);
+            const bool t = in && !(need <= T.gamma * lbv);
+            const unsigned m = g.ballot(t);
+            float nl = lbv - need;
+            if (t) {
+                const int pos = nlist + __popc(m & ((1u << g.sl) - 1u));
+                sc.pair[pos] = (short)(b | ((acc.exact >> s) & 1u ? 0x4000 : 0));
+                sc.dist[pos] = lbv;
+                nl = __int_as_float(pos);
+                trig |= 1u << s;
+            }
+            acc.lb[s] = nl;
+            nlist += __popc(m);
+        };
+        {
+            // link and box of the lane's pair, stepped by LPS pairs a pass
+            const int dl = nb > 0 ? LPS / nb : 0, db = LPS - dl * nb;
+            int l = nb > 0 ? g.sl / nb : 0, bx = g.sl - l * nb;
+#pragma unroll 1
+            for (int s = 0; s < ncb; ++s) {
+                const int b = g.sl + LPS * s;
+                const bool in = b < nlb;
+                screen(s, b, in, sc.motion[in ? l : 0]);
+                l += dl;
+                bx += db;
+                if (bx >= nb) {
+                    bx -= nb;
+                    ++l;
+                }
+            }
+        }
+        const int nbox = nlist;
+#pragma unroll 1
+        for (int s = 0; s < td::CC; ++s) {
+            const int b = g.sl + LPS * s;
+            const bool in = b < ncc, ball = b < nball;
+            const int r = in && !ball ? b - nball : 0, i = r / NA, j = r - i * NA;
+            screen(td::CB + s, b, in, ball ? sc.motion[in ? b : 0] + mb : sc.motion[i] + sc.motion[NA + j]);
+        }
+        acc.exact = trig;
+        g.sync();
+        // entry e of the list is slot e % 32's, whatever LPS is
+        auto add = [&](int e, float d0, float d1) {
+            const float v = fmaxf(-d1 + keep * d0, 0.0f) + (d1 < 0.0f ? 1.0f : 0.0f);
+            const int ps = (e / LPS) & (PS - 1);
+#pragma unroll
+            for (int t = 0; t < PS; ++t) acc.c[t] += ps == t ? v : 0.0f;
+            sc.dist[e] = d1;
+        };
+#pragma unroll 1
+        for (int e = g.sl; e < nbox; e += LPS) {
+            const int en = sc.pair[e], b = en & 0x3fff;
+            const int l = b / nb, bx = b - l * nb;
+            const float rc = M.link[l / NA][l % NA].rcap;
+            float d0 = sc.dist[e], d1 = 0.0f;
+#pragma unroll 1
+            for (int now = en & 0x4000 ? 1 : 0; now < 2; ++now) {  // one copy of the distance's code
+                d1 = capsule_box_distance(now ? &w.a0[l][0] : &pv.a[l][0], now ? &w.a1[l][0] : &pv.a[l][3], rc, M.box[bx]);
+                d0 = now ? d0 : d1;
+            }
+            add(e, d0, d1);
+        }
+#pragma unroll 1
+        for (int e = nbox + ((g.sl - nbox) & (LPS - 1)); e < nlist; e += LPS) {
+            const int en = sc.pair[e], b = en & 0x3fff;
+            float d0 = sc.dist[e], d1 = 0.0f;
+#pragma unroll 1
+            for (int now = en & 0x4000 ? 1 : 0; now < 2; ++now) {
+                d1 = segment_pair(b, now != 0);
+                d0 = now ? d0 : d1;
+            }
+            add(e, d0, d1);
+        }
+        g.sync();
+        while (trig) {  // the listed pairs' distances back to their lanes
+            const int s = __ffs(trig) - 1;
+            trig &= trig - 1u;
+            acc.lb[s] = sc.dist[__float_as_int(acc.lb[s])];
         }
     }
-    // ball-link and link-link passes (the ball is a capsule of zero length)
+    if (g.sl < 2 * NA) {
 #pragma unroll
-    for (int s = 0; s < TaskDims<NA>::CC; ++s) {
-        const int b = lane + 32 * s;
-        if (b < ncc) {
-            const bool ball = b < nball;
-            const int r = b - nball, i = r / NA, j = r - i * NA;
-            const int la = ball ? b : i, lb = ball ? 0 : NA + j;
-            const float* c0 = ball ? &w.q[d::B] : w.a0[lb];
-            const float* c1 = ball ? &w.q[d::B] : w.a1[lb];
-            const float rb = ball ? M.rb : M.link[1][j].rcap;
-            const float dist = capsule_capsule_distance(w.a0[la], w.a1[la], M.link[la / NA][la % NA].rcap, c0, c1, rb);
-            if (!first) acc.c += fmaxf(-dist + keep * acc.prevc[s], 0.0f) + (dist < 0.0f ? 1.0f : 0.0f);
-            acc.prevc[s] = dist;
+        for (int k = 0; k < 3; ++k) {
+            pv.a[g.sl][k] = w.a0[g.sl][k];
+            pv.a[g.sl][3 + k] = w.a1[g.sl][k];
         }
     }
-    if (first) return;
+    if (g.sl < 3) pv.ball[g.sl] = w.q[d::B + g.sl];
+    if (first) {
+        g.sync();
+        return;
+    }
     // end effectors: velocity = sum over the arm's joints of (z_j x (p - o_j)) qd_j
-    const int a = lane >> 4, i = lane & 15;
+    const int a = g.a, i = g.i;
     const float* pe = w.a1[a * NA + NA - 1];
     float vx = 0.0f, vy = 0.0f, vz = 0.0f;
     if (i < NA) {
@@ -303,10 +436,10 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
         vz = (z[0] * r1 - z[1] * r0) * qdj;
     }
 #pragma unroll
-    for (int off = 8; off > 0; off >>= 1) {
-        vx += __shfl_xor_sync(FULL, vx, off);
-        vy += __shfl_xor_sync(FULL, vy, off);
-        vz += __shfl_xor_sync(FULL, vz, off);
+    for (int off = Lanes<LPS>::SEG / 2; off > 0; off >>= 1) {
+        vx += g.xor_(vx, off);
+        vy += g.xor_(vy, off);
+        vz += g.xor_(vz, off);
     }
     if (i == NA - 1) {
         float* e = w.ee[a];
@@ -322,14 +455,13 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
         acc.r += 0.5f * quat_angle(qe, a == 0 ? T.q1s : T.q2s);
     }
     float th = 0.0f;
-    if (lane < d::NU) {
-        const float e = w.q[lane] - T.home[lane];
+    if (g.sl < d::NU) {
+        const float e = w.q[g.sl] - T.home[g.sl];
         th = e * e;
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) th += __shfl_xor_sync(FULL, th, off);
-    __syncwarp();
-    if (lane == 0) {
+    th = group_sum(g, th);
+    g.sync();
+    if (g.sl == 0) {
         const float* e1 = w.ee[0];
         const float* e2 = w.ee[1];
         const float dp0 = e1[0] - e2[0], dp1 = e1[1] - e2[1], dp2 = e1[2] - e2[2];
@@ -345,19 +477,14 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
         const float t0 = c0 - T.ptg[0], t1 = c1 - T.ptg[1], t2 = c2 + T.eps - T.ptg[2];
         acc.ot += sqrtf(t0 * t0 + t1 * t1 + t2 * t2);
     }
-    __syncwarp();
+    g.sync();
 }
 
 // Weighted total after the last state (the barrier and orientation sums
-// reduced over the warp; the other terms from lane 0).
-template <int NA>
-__device__ __forceinline__ float task_total(const DevTask& T, TaskAcc<NA>& acc) {
-    float c = acc.c, r = acc.r;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        c += __shfl_xor_sync(FULL, c, off);
-        r += __shfl_xor_sync(FULL, r, off);
-    }
+// reduced over the group; the other terms from lane 0).
+template <int NA, int LPS>
+__device__ __forceinline__ float task_total(const DevTask& T, const Lanes<LPS>& g, TaskAcc<NA, LPS>& acc) {
+    const float c = slot_sum(g, acc.c), r = group_sum(g, acc.r);
     const float pick = T.phase == 0 ? 1.0f : 0.0f, move = 1.0f - pick;
     return pick * (T.w_c * c + T.w_eo * acc.eo) + move * (T.w_c * c + T.w_ot * acc.ot) + T.w_theta * acc.th +
            T.w_yz * acc.yz + T.w_v * sqrtf(acc.v2) + T.w_r * r + T.w_l * acc.l;
