@@ -18,20 +18,19 @@ struct __align__(16) DevTask {
     float home[16];        // theta_home
 };
 
-// pairs: links x boxes (link-major) in the first lane passes, then links x
-// ball (pick) and left x right links, so that every pass holds one kind
+// pairs: links x boxes (link-major; link l is lane l's), then links x ball
+// (pick) and left x right links, one pair per lane and pass
 template <int NA, int LPS>
 struct TaskDims {
-    static constexpr int CB = (2 * NA * MAXB + LPS - 1) / LPS;  // capsule-box passes at most
-    static constexpr int CC = (2 * NA + NA * NA + LPS - 1) / LPS;
-    static_assert(CB + CC <= 32, "one bit per pass");
+    static constexpr int CC = (2 * NA + NA * NA + LPS - 1) / LPS;  // passes of the second kind at most
 };
 
 template <int NA, int LPS>
 struct TaskAcc {
-    // this lane's pairs, one per pass: a lower bound of the pair's distance at
-    // the previous state, the distance itself where the bit of exact is set
-    float lb[TaskDims<NA, LPS>::CB + TaskDims<NA, LPS>::CC];
+    // lower bounds at the previous state: of this lane's link's distance to any
+    // box, and of its pairs' distances in the passes -- the distance itself
+    // where the bit of exact is set
+    float lbox, lb[TaskDims<NA, LPS>::CC];
     unsigned exact;
     float c[32 / LPS];              // barrier + penetration count, per slot of the pair list
     float r;                        // orientation error (the end-effector lanes)
@@ -262,21 +261,23 @@ __device__ __forceinline__ float quat_angle(const float* q, const float* qs) {
 // previous one (gamma < 1, so a penetrating pair always does).  A distance
 // changes by at most the motion of the pair's ends, so a pair whose lower bound
 // at the previous state is above motion / gamma adds nothing: its bound drops by
-// the motion and no distance is formed.  The others (near or fast ones, a few of
-// up to 287) go to a list in pair order, spread over the group's lanes, each
-// with its distance now and, unless that is known from the previous state, the
-// one before.  The margins (1e-5 of the motion, 2e-5 m) are far above the
-// rounding of the distances, so the terms are those of testing every pair.
-// MEASURED_TASK
+// the motion and no distance is formed.  The others (near or fast ones) go to a
+// list in pair order, spread over the group's lanes, each with its distance now
+// and, unless that is known from the previous state, the one before.  Link-box
+// pairs share one bound per link (a link that fails puts all its boxes on the
+// list; on the transfer 0.04 pairs a state need their distance, of 112): bounds
+// per pair took the lane's local memory.  The margins (1e-5 of the motion,
+// 2e-5 m) are far above the rounding of the distances, so the terms are those of
+// testing every pair.  One iteration of the transfer with the suite (K = 4096, H =
+// 64): 1,360 us with every distance on 32 lanes, 800 screened per pair (16
+// lanes), 525 with the bound per link.
 template <int NA, int LPS>
 __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, WarpWS<NA>& w, const Lanes<LPS>& g,
                                            const float (&Rl)[9], bool first, TaskAcc<NA, LPS>& acc) {
     using d = Dims<NA>;
-    using td = TaskDims<NA, LPS>;
-    constexpr int PS = 32 / LPS;
+    constexpr int CC = TaskDims<NA, LPS>::CC, PS = 32 / LPS;
     TaskPrev<NA>& pv = *reinterpret_cast<TaskPrev<NA>*>(&w + 1);
     const int nb = M.nb, nlb = 2 * NA * nb;
-    const int ncb = (nlb + LPS - 1) / LPS;  // capsule-box passes
     const int nball = T.phase == 0 ? 2 * NA : 0;
     const int ncc = nball + NA * NA;
     const float keep = 1.0f - T.gamma;
@@ -291,25 +292,24 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
         const float* c1 = ball ? c0 : (now ? &w.a1[lb][0] : &pv.a[lb][3]);
         return capsule_capsule_distance(x0, x1, M.link[la / NA][la % NA].rcap, c0, c1, ball ? M.rb : M.link[1][j].rcap);
     };
+    auto& sc = w.ph.task;
+    const bool own = g.sl < 2 * NA;  // this lane has a link
     if (first) {
 #pragma unroll 1
-        for (int s = 0; s < ncb; ++s) {
-            const int b = g.sl + LPS * s;
-            if (b < nlb) {
-                const int l = b / nb, bx = b - l * nb;
-                acc.lb[s] = capsule_box_distance(w.a0[l], w.a1[l], M.link[l / NA][l % NA].rcap, M.box[bx]);
-            }
+        for (int b = g.sl; b < nlb; b += LPS) {
+            const int l = b / nb, bx = b - l * nb;
+            sc.dist[b] = capsule_box_distance(w.a0[l], w.a1[l], M.link[l / NA][l % NA].rcap, M.box[bx]);
         }
-#pragma unroll 1
-        for (int s = 0; s < td::CC; ++s) {
-            const int b = g.sl + LPS * s;
-            if (b < ncc) acc.lb[td::CB + s] = segment_pair(b, true);
-        }
+        g.sync();
+        acc.lbox = INFINITY;
+        for (int bx = 0; bx < nb && own; ++bx) acc.lbox = fminf(acc.lbox, sc.dist[g.sl * nb + bx]);
+#pragma unroll
+        for (int s = 0; s < CC; ++s) acc.lb[s] = g.sl + LPS * s < ncc ? segment_pair(g.sl + LPS * s, true) : 0.0f;
         acc.exact = ~0u;
     } else {
-        auto& sc = w.ph.task;
         // motion of every link's ends and of the ball since the previous state
-        if (g.sl < 2 * NA) {
+        float ml = 0.0f;
+        if (own) {
             float m0 = 0.0f, m1 = 0.0f;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
@@ -317,7 +317,8 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
                 m0 = __fmaf_rn(e0, e0, m0);
                 m1 = __fmaf_rn(e1, e1, m1);
             }
-            sc.motion[g.sl] = sqrtf(fmaxf(m0, m1));
+            ml = sqrtf(fmaxf(m0, m1));
+            sc.motion[g.sl] = ml;
         }
         float mb = 0.0f;
 #pragma unroll
@@ -327,16 +328,36 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
         }
         mb = sqrtf(mb);
         g.sync();
+        const auto need = [](float motion) { return __fmaf_rn(motion, 1.00001f, 2e-5f); };
+        const unsigned below = (1u << g.sl) - 1u;
         int nlist = 0;
+        bool tbox = false;  // this lane's link meets its bound
+        int pbox = 0;
+        if (nb > 0) {
+            const float nd = need(ml);
+            tbox = own && !(nd <= T.gamma * acc.lbox);
+            acc.lbox -= nd;
+            const unsigned m = g.ballot(tbox);
+            if (m) {
+                pbox = nb * __popc(m & below);
+                nlist = nb * __popc(m);
+                for (int bx = 0; bx < nb && tbox; ++bx) sc.pair[pbox + bx] = (short)(g.sl * nb + bx);
+            }
+        }
+        const int nbox = nlist;
         unsigned trig = 0u;
-        // a pair of pass bit s: screened, or put on the list with its bound
-        auto screen = [&](int s, int b, bool in, float motion) {
-            const float lbv = acc.lb[s], need = __fmaf_rn(motion, 1.00001f, 2e-5f);
-            const bool t = in && !(need <= T.gamma * lbv);
+#pragma unroll
+        for (int s = 0; s < CC; ++s) {
+            const int b = g.sl + LPS * s;
+            const bool in = b < ncc, ball = b < nball;
+            const int r = in && !ball ? b - nball : 0, i = r / NA, j = r - i * NA;
+            const float nd = need(ball ? sc.motion[in ? b : 0] + mb : sc.motion[i] + sc.motion[NA + j]);
+            const float lbv = acc.lb[s];
+            const bool t = in && !(nd <= T.gamma * lbv);
             const unsigned m = g.ballot(t);
-            float nl = lbv - need;
+            float nl = lbv - nd;
             if (t) {
-                const int pos = nlist + __popc(m & ((1u << g.sl) - 1u));
+                const int pos = nlist + __popc(m & below);
                 sc.pair[pos] = (short)(b | ((acc.exact >> s) & 1u ? 0x4000 : 0));
                 sc.dist[pos] = lbv;
                 nl = __int_as_float(pos);
@@ -344,31 +365,6 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
             }
             acc.lb[s] = nl;
             nlist += __popc(m);
-        };
-        {
-            // link and box of the lane's pair, stepped by LPS pairs a pass
-            const int dl = nb > 0 ? LPS / nb : 0, db = LPS - dl * nb;
-            int l = nb > 0 ? g.sl / nb : 0, bx = g.sl - l * nb;
-#pragma unroll 1
-            for (int s = 0; s < ncb; ++s) {
-                const int b = g.sl + LPS * s;
-                const bool in = b < nlb;
-                screen(s, b, in, sc.motion[in ? l : 0]);
-                l += dl;
-                bx += db;
-                if (bx >= nb) {
-                    bx -= nb;
-                    ++l;
-                }
-            }
-        }
-        const int nbox = nlist;
-#pragma unroll 1
-        for (int s = 0; s < td::CC; ++s) {
-            const int b = g.sl + LPS * s;
-            const bool in = b < ncc, ball = b < nball;
-            const int r = in && !ball ? b - nball : 0, i = r / NA, j = r - i * NA;
-            screen(td::CB + s, b, in, ball ? sc.motion[in ? b : 0] + mb : sc.motion[i] + sc.motion[NA + j]);
         }
         acc.exact = trig;
         g.sync();
@@ -382,12 +378,11 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
         };
 #pragma unroll 1
         for (int e = g.sl; e < nbox; e += LPS) {
-            const int en = sc.pair[e], b = en & 0x3fff;
-            const int l = b / nb, bx = b - l * nb;
+            const int b = sc.pair[e], l = b / nb, bx = b - l * nb;
             const float rc = M.link[l / NA][l % NA].rcap;
-            float d0 = sc.dist[e], d1 = 0.0f;
+            float d0 = 0.0f, d1 = 0.0f;
 #pragma unroll 1
-            for (int now = en & 0x4000 ? 1 : 0; now < 2; ++now) {  // one copy of the distance's code
+            for (int now = 0; now < 2; ++now) {  // one copy of the distance's code
                 d1 = capsule_box_distance(now ? &w.a0[l][0] : &pv.a[l][0], now ? &w.a1[l][0] : &pv.a[l][3], rc, M.box[bx]);
                 d0 = now ? d0 : d1;
             }
@@ -405,13 +400,16 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
             add(e, d0, d1);
         }
         g.sync();
-        while (trig) {  // the listed pairs' distances back to their lanes
-            const int s = __ffs(trig) - 1;
-            trig &= trig - 1u;
-            acc.lb[s] = sc.dist[__float_as_int(acc.lb[s])];
+        // the listed pairs' distances back to their lanes
+        if (tbox) {
+            acc.lbox = INFINITY;
+            for (int bx = 0; bx < nb; ++bx) acc.lbox = fminf(acc.lbox, sc.dist[pbox + bx]);
         }
+#pragma unroll
+        for (int s = 0; s < CC; ++s)
+            if ((trig >> s) & 1u) acc.lb[s] = sc.dist[__float_as_int(acc.lb[s])];
     }
-    if (g.sl < 2 * NA) {
+    if (own) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             pv.a[g.sl][k] = w.a0[g.sl][k];
