@@ -339,12 +339,12 @@ int mppi_set_launch(mppi_ctx *c, int samples_per_cta);
 
 /* Layout of the rollout kernels.  lanes_per_sample: 32 (one sample per
  * warp), 16 (two) or 8 (four; 3-link arms only); 0 = 32.  The default of a
- * new controller is 16 when K exceeds 16 x the SM count (32-lane groups'
- * registers then cannot hold all samples at once), else 32.  placement of the
+ * new controller is 16 when K exceeds 8 x the SM count (16 x for 3-link
+ * arms), else 32.  placement of the
  * solve of a lone ball contact with static geometry: 0 = fused with the
  * arms' factorisation (every lane runs both chains), 1 = after it.  Every
  * layout gives bitwise the same samples, costs and updates.  The ball-task
- * cost suite always runs on 32 lanes per sample.  Errors:
+ * cost suite runs on 32 lanes where 8 are set, and with the fused placement.  Errors:
  * MPPI_ERR_INVALID_ARG for other values or more than 512 threads per CTA,
  * MPPI_ERR_UNSUPPORTED for 8 lanes with 7-link arms. */
 int mppi_set_layout(mppi_ctx *c, int lanes_per_sample, int placement);
@@ -394,7 +394,10 @@ const float *mppi_batch_costs(const mppi_batch *b, int i);
 int mppi_batch_set_launch(mppi_batch *b, int samples_per_cta, int order);
 int mppi_batch_get_launch(const mppi_batch *b, int *samples_per_cta, int *order);
 /* Layout: lanes per sample (32, 16, or 8 for 3-link arms; 0 = 32) and the
- * placement of the lone ball contact's solve (as mppi_set_layout). */
+ * placement of the lone ball contact's solve (as mppi_set_layout).  A new
+ * batch has the layout that its total number of samples gives a controller
+ * (16 lanes with 2 or 16 samples per CTA, else 32 with 4) unless a tuned
+ * choice is stored for it. */
 int mppi_batch_set_layout(mppi_batch *b, int lanes_per_sample, int placement);
 int mppi_batch_get_layout(const mppi_batch *b, int *lanes_per_sample, int *placement);
 /* Autotuner: times `reps` iterations of every shape -- lanes per sample

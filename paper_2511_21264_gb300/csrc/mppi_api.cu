@@ -452,7 +452,7 @@ int mppi_create(const mppi_model* m, int K, int H, float lambda, const float* si
     c->lambda = lambda;
     c->seed = seed;
     c->n_elite = K;
-    c->lps = default_lps(K);
+    c->lps = default_lps(m->info.na, K);
     c->spc = default_spc(c);
     const int nu = 2 * m->info.na;
     std::vector<float> lo(nu), hi(nu);

@@ -593,6 +593,17 @@ int mppi_batch_create(const mppi_batch_desc* desc, int n, mppi_batch** out) {
     std::snprintf(key, sizeof key, "nv%d_nb%d_n%d_K%lld_H%d", 2 * na + 6, boxes <= 0 ? 0 : (boxes <= 8 ? 8 : 16), n,
                   ksum, b->max_h);
     b->key = key;
+    // without a stored choice: a single controller's layout for the batch's
+    // samples; on 16 lanes the widest CTAs once the samples fill every SM (32
+    // each), one-warp CTAs below, which spread evenly.  One GB300, ms: 64
+    // controllers of the configurations' pool 7.3 on 32 lanes with 4 samples per
+    // CTA, 5.5 / 5.1 / 4.6 / 4.5 on 16 with 2 / 4 / 8 / 16; 5 controllers (5632
+    // samples) 0.45, and 0.31 / 0.32 / 0.30 / 0.28; 2 (3072 samples) 0.46, and
+    // 0.44 / 0.51 / 0.51 / 0.49
+    if (default_lps(na, ksum) == 16) {
+        b->lps = 16;
+        b->spc = ksum > 32LL * sm_count() ? 16 : 2;
+    }
     int spc = 0, order = 0, lps = 0, place = 0;
     if (mppi_tune_lookup(key, &spc, &order, &lps, &place) == MPPI_OK) {
         b->spc = spc;

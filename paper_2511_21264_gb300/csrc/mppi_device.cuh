@@ -153,11 +153,18 @@ struct __align__(16) WarpWS {
     CArr<float, d::NV> rhs;
     CArr<float, d::NU> u;
     CArr<CArr<float, 16>, 8> zn;  // standard normals of the next steps (Philox path)
-    // kinematics, per link (read across lanes)
-    CArr<CArr<float, 3>, d::NL> z;
-    CArr<CArr<float, 3>, d::NL> o;
-    CArr<CArr<float, 3>, d::NL> a0;
-    CArr<CArr<float, 3>, d::NL> a1;
+    // kinematics, per link (read across lanes), until the contact rows are
+    // formed; then the Delassus block.  With the block in storage of its own a
+    // batch's SM held 24 samples (12 warps) instead of 32
+    union {
+        struct {
+            CArr<CArr<float, 3>, d::NL> z;
+            CArr<CArr<float, 3>, d::NL> o;
+            CArr<CArr<float, 3>, d::NL> a0;
+            CArr<CArr<float, 3>, d::NL> a1;
+        };
+        CArr<float, 9 * MAXC * MAXC> G;  // entry (3 c + k, 3 q + m) at ((9 q + 3 k + m) MAXC + c), R added on the diagonal
+    };
     // factors of (M + dt D), per arm
     CArr<CArr<CArr<float, NA>, NA>, 2> L;
     CArr<CArr<float, NA>, 2> Ldi;  // reciprocal diagonal of the factors
@@ -167,14 +174,12 @@ struct __align__(16) WarpWS {
     CArr<float, MAXC> cdep;
     CArr<int, MAXC> cA;
     CArr<int, MAXC> cB;
-    CArr<CArr<float, 6>, 2> ee;   // task cost: end-effector position and velocity per arm
     union Phase {
         struct {
             CArr<short, 2 * MAXL * MAXB> surv;  // capsule-box pairs that pass the cull
         } col;
         struct {
             CArr<CArr<float4, (d::NV + 3) / 4>, MAXR> Y;  // half-solved rows, zero-padded to whole float4s
-            CArr<float, 9 * MAXC * MAXC> G;  // Delassus entry (3 c + k, 3 q + m) at ((9 q + 3 k + m) MAXC + c), R added on the diagonal
             CArr<float, MAXR> rho;       // per row: b - reference velocity, with b = J v_f
             CArr<float, MAXR> iA;        // 1 / (A + R)
             CArr<float, MAXR> lam;
@@ -1369,9 +1374,13 @@ __device__ __forceinline__ void pgs_sweeps(const DevModel& M, WarpWS<NA>& w, con
         rho[k] = w.ph.con.rho[3 * c + k];
         iA[k] = w.ph.con.iA[3 * c + k];
         lam[k] = 0.0f;
-        if (k) Gd[k - 1] = w.ph.con.G[(9 * c + 3 * k) * MAXC + c];
+        if (k) Gd[k - 1] = w.G[(9 * c + 3 * k) * MAXC + c];
     }
     const float mu = M.mu;
+    auto block = [&](int q, float (&Gq)[9]) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) Gq[k] = w.G[(9 * q + k) * MAXC + c];
+    };
     auto contact = [&](int q, const float (&Gq)[9]) {
         const float ln = fmaxf(__fmaf_rn(-rho[0], iA[0], lam[0]), 0.0f), dn = ln - lam[0];
         float l1 = __fmaf_rn(-__fmaf_rn(Gd[0], dn, rho[1]), iA[1], lam[1]);
@@ -1393,8 +1402,7 @@ __device__ __forceinline__ void pgs_sweeps(const DevModel& M, WarpWS<NA>& w, con
         float Gq[NC][9];
 #pragma unroll
         for (int q = 0; q < NC; ++q)
-#pragma unroll
-            for (int k = 0; k < 9; ++k) Gq[q][k] = q < nc ? w.ph.con.G[(9 * q + k) * MAXC + c] : 0.0f;
+            block(q < nc ? q : 0, Gq[q]);
         for (int sw = 0; sw < M.sweeps; ++sw) {
 #pragma unroll
             for (int q = 0; q < NC; ++q)
@@ -1404,8 +1412,7 @@ __device__ __forceinline__ void pgs_sweeps(const DevModel& M, WarpWS<NA>& w, con
         for (int sw = 0; sw < M.sweeps; ++sw)
             for (int q = 0; q < nc; ++q) {
                 float Gq[9];
-#pragma unroll
-                for (int k = 0; k < 9; ++k) Gq[k] = w.ph.con.G[(9 * q + k) * MAXC + c];
+                block(q, Gq);
                 contact(q, Gq);
             }
     }
@@ -1557,7 +1564,7 @@ __device__ __forceinline__ void contacts(const DevModel& M, WarpWS<NA>& w, const
                 const bool dia = 3 * q + m == r;
                 gv = dia ? __fmaf_rn(regc, gv, gv) : gv;  // A + R, R = regc A
                 gd = dia ? gv : gd;
-                w.ph.con.G[(9 * q + 3 * k + m) * MAXC + c] = gv;
+                w.G[(9 * q + 3 * k + m) * MAXC + c] = gv;
             }
         }
         w.ph.con.iA[r] = 1.0f / gd;

@@ -250,15 +250,25 @@ bool task_fits(int spc, int unom_floats) {
            rollout_smem<NA, 16, true>((spc + 1) / 2 * 2, unom_floats) <= (size_t)max_sm;
 }
 
-// Default layout for K samples: 16 lanes per sample once 32-lane groups
-// cannot hold all K samples in one wave (their registers allow 16 warps per
-// SM), else 32 (the shorter per-step chain of one sample per warp).
-inline int default_lps(int K) {
+// SMs of the current device, 0 if unknown.
+inline int sm_count() {
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0)
-        return 32;
-    return K > 16 * nsm ? 16 : 32;
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    return nsm;
+}
+
+// Default layout for K samples: 16 lanes per sample once 32-lane groups would
+// take more than 8 warps per SM (7-link arms; 16 for the shorter 3-link steps,
+// where 32-lane groups can no longer hold all samples at once), else 32 (the
+// shorter per-step chain of one sample per warp).  One GB300, us per iteration
+// on 32 / 16 lanes: transfer H = 64, K = 1216 205 / 242, K = 2048 284 / 246,
+// K = 2432 288 / 270; lift H = 32, K = 1216 89 / 90, K = 2048 128 / 102;
+// planar H = 20, K = 2048 125 / 126, K = 4096 236 / 151.
+inline int default_lps(int na, long long K) {
+    const int nsm = sm_count();
+    return nsm > 0 && K > (na == 7 ? 8LL : 16LL) * nsm ? 16 : 32;
 }
 
 int launch_rollout_na7(int mode, const RolloutArgs& a, int spc, cudaStream_t s);

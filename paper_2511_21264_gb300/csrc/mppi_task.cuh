@@ -37,11 +37,13 @@ struct TaskAcc {
     float th, yz, v2, l, eo, ot;    // per-state terms (lane 0)
 };
 
-// The previous state's capsule ends and ball, behind the sample's workspace.
+// The previous state's capsule ends and ball, and the end effectors' positions
+// and velocities, behind the sample's workspace.
 template <int NA>
 struct __align__(16) TaskPrev {
     CArr<CArr<float, 6>, 2 * NA> a;
     CArr<float, 4> ball;
+    CArr<CArr<float, 6>, 2> ee;
 };
 
 // Minimum over t in [0,1] of the box SDF f(t) at a0 + t dd, for any segment
@@ -440,7 +442,7 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
         vz += g.xor_(vz, off);
     }
     if (i == NA - 1) {
-        float* e = w.ee[a];
+        float* e = pv.ee[a];
         e[0] = pe[0];
         e[1] = pe[1];
         e[2] = pe[2];
@@ -460,8 +462,8 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
     th = group_sum(g, th);
     g.sync();
     if (g.sl == 0) {
-        const float* e1 = w.ee[0];
-        const float* e2 = w.ee[1];
+        const float* e1 = pv.ee[0];
+        const float* e2 = pv.ee[1];
         const float dp0 = e1[0] - e2[0], dp1 = e1[1] - e2[1], dp2 = e1[2] - e2[2];
         const float rv = dp0 * (e1[3] - e2[3]) + dp1 * (e1[4] - e2[4]) + dp2 * (e1[5] - e2[5]);
         const float c0 = 0.5f * (e1[0] + e2[0]), c1 = 0.5f * (e1[1] + e2[1]), c2 = 0.5f * (e1[2] + e2[2]);
