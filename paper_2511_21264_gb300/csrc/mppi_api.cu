@@ -58,6 +58,8 @@ __global__ void noise_kernel(NoiseArgs a) {
 // mppi_kernels.cuh).
 __global__ void __launch_bounds__(1024) elite_select_kernel(const float* costs, int K, int P, int n_elite,
                                                             unsigned long long* sel, int* eidx) {
+    cudaGridDependencySynchronize();  // the rollout's costs
+    cudaTriggerProgrammaticLaunchCompletion();
     extern __shared__ unsigned long long keys[];
     __shared__ int nfin;
     elite_select_block(costs, K, P, n_elite, sel, eidx, keys, nfin);
@@ -65,6 +67,7 @@ __global__ void __launch_bounds__(1024) elite_select_kernel(const float* costs, 
 
 template <int NU>
 __global__ void __launch_bounds__(256) elite_update_kernel(EliteArgs a) {
+    cudaGridDependencySynchronize();  // the elite list
     __shared__ EliteSmem<NU> sm;
     elite_update_step<NU>(a, blockIdx.x, sm);
     if (a.advance) {
@@ -746,7 +749,7 @@ int qp_build(int nu, int K, int H, const float* bounds, float rho, const float* 
         if (rc != MPPI_OK) return rc;
     }
     if (H > MPPI_QP_MAX_H) return MPPI_ERR_UNSUPPORTED;
-    const int L = qp_lanes(K * nu, H);
+    const int L = qp_lanes(K * nu, H, true);
     const size_t per = (size_t)qp_table_size(H, L) * sizeof(float4);
     std::vector<QPClass> cls(nu);
     *n_tab = 1;
@@ -776,7 +779,7 @@ QPArgs qp_controller_args(int nu, int nq, int K, int H, int iters, float dt, con
     q.iters = iters;
     q.per_cls = K;
     q.dt = dt;
-    q.L = qp_lanes(q.n, H);
+    q.L = qp_lanes(q.n, H, true);
     q.tab_size = qp_table_size(H, q.L);
     q.n_tab = n_tab;
     q.cls = static_cast<const QPClass*>(d_qp);
@@ -893,7 +896,7 @@ static bool elite_mode(const mppi_ctx* c) {
 }
 
 static int launch_elite(mppi_ctx* c, const float* costs, const float* u_nom, float* u_out, int advance,
-                        const float* U_stored, cudaStream_t s) {
+                        const float* U_stored, bool pdl, cudaStream_t s) {
     const int nu = 2 * c->m->info.na;
     int P = 1;
     while (P < c->K) P <<= 1;
@@ -904,8 +907,10 @@ static int launch_elite(mppi_ctx* c, const float* costs, const float* u_nom, flo
         cudaError_t e = cudaFuncSetAttribute(elite_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return cuda_fail(e);
     }
-    elite_select_kernel<<<1, 1024, sm, s>>>(costs, c->K, P, c->n_elite, c->d_sel, c->d_eidx);
-    cudaError_t e = cudaGetLastError();
+    // both kernels as programmatic dependents: their launches overlap the tails
+    // of the rollout and of the selection
+    cudaError_t e = launch_kernel(elite_select_kernel, dim3(1), dim3(1024), sm, s, pdl, costs, c->K, P, c->n_elite,
+                                  c->d_sel, c->d_eidx);
     if (e != cudaSuccess) return cuda_fail(e);
     EliteArgs a{};
     a.K = c->K;
@@ -933,9 +938,9 @@ static int launch_elite(mppi_ctx* c, const float* costs, const float* u_nom, flo
     a.err = c->d_err;
     a.advance = advance;
     a.done = c->d_done;
-    if (nu == 6) elite_update_kernel<6><<<c->H, 256, 0, s>>>(a);
-    else elite_update_kernel<14><<<c->H, 256, 0, s>>>(a);
-    return cuda_fail(cudaGetLastError());
+    if (nu == 6) e = launch_kernel(elite_update_kernel<6>, dim3(c->H), dim3(256), 0, s, pdl, a);
+    else e = launch_kernel(elite_update_kernel<14>, dim3(c->H), dim3(256), 0, s, pdl, a);
+    return cuda_fail(e != cudaSuccess ? e : cudaGetLastError());
 }
 
 static UpdateArgs update_args(mppi_ctx* c, const float* costs, const float* u_nom, float* u_out, int advance,
@@ -991,7 +996,7 @@ static int enqueue_step(mppi_ctx* c, const float* state, const float* u_nom, flo
     if (rc != MPPI_OK) return rc;
     if (prof) cudaEventRecord(ev[2], s);
     if (elite_mode(c)) {
-        rc = launch_elite(c, c->d_costs, u_nom, u_out, 1, c->d_U, s);
+        rc = launch_elite(c, c->d_costs, u_nom, u_out, 1, c->d_U, pdl, s);
     } else {
         UpdateArgs u = update_args(c, c->d_costs, u_nom, u_out, 1, best);
         u.U_stored = c->d_U;
@@ -1088,7 +1093,7 @@ int mppi_solve(mppi_ctx* c, const float* state, float* u, int iters, float* best
 
 int mppi_update(mppi_ctx* c, const float* costs, const float* u_nom, float* u_out, void* stream) {
     if (!c || !costs || !u_nom || !u_out) return MPPI_ERR_INVALID_ARG;
-    if (elite_mode(c)) return launch_elite(c, costs, u_nom, u_out, 0, nullptr, (cudaStream_t)stream);
+    if (elite_mode(c)) return launch_elite(c, costs, u_nom, u_out, 0, nullptr, false, (cudaStream_t)stream);
     UpdateArgs u = update_args(c, costs, u_nom, u_out, 0, c->d_best);
     return launch_update(2 * c->m->info.na, u, c->H, (cudaStream_t)stream);
 }

@@ -165,6 +165,7 @@ struct __align__(16) WarpWS {
         };
         CArr<float, 9 * MAXC * MAXC> G;  // entry (3 c + k, 3 q + m) at ((9 q + 3 k + m) MAXC + c), R added on the diagonal
     };
+    CArr<CArr<float, 6>, d::NL> ref;  // every link's capsule ends at the last cull against the boxes
     // factors of (M + dt D), per arm
     CArr<CArr<CArr<float, NA>, NA>, 2> L;
     CArr<CArr<float, NA>, 2> Ldi;  // reciprocal diagonal of the factors
@@ -303,21 +304,16 @@ __device__ __forceinline__ void forward_kinematics(const DevModel& M, WarpWS<NA>
         p[1] = sn * L.Fp[0] + cs * L.Fp[1];
         p[2] = L.Fp[2];
     }
-    // the lanes past the last link hold the identity through all rounds, and a
-    // lane with no predecessor this far back takes it from there: no selects
-    // on the products (24 of about 2,000 instructions of a step)
-#pragma unroll
-    for (int k = 0; k < 9; ++k) R[k] = act ? R[k] : (k % 4 == 0 ? 1.0f : 0.0f);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) p[k] = act ? p[k] : 0.0f;
 #pragma unroll
     for (int off = 1; off < NA; off <<= 1) {
-        const int src = act && i >= off ? i - off : NA;
         float Rp[9], pp[3];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) Rp[k] = g.from_seg(R[k], src);
+        for (int k = 0; k < 9; ++k) Rp[k] = g.up_seg(R[k], off);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) pp[k] = g.from_seg(p[k], src);
+        for (int k = 0; k < 3; ++k) pp[k] = g.up_seg(p[k], off);
+        // every lane forms the product; lanes with no predecessor this far
+        // back keep their transform (a select, no divergent branch)
+        const bool take = i >= off;
         float Rn[9], pn[3];
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
@@ -327,9 +323,9 @@ __device__ __forceinline__ void forward_kinematics(const DevModel& M, WarpWS<NA>
             pn[r] = Rp[3 * r] * p[0] + Rp[3 * r + 1] * p[1] + Rp[3 * r + 2] * p[2] + pp[r];
         }
 #pragma unroll
-        for (int k = 0; k < 9; ++k) R[k] = Rn[k];
+        for (int k = 0; k < 9; ++k) R[k] = take ? Rn[k] : R[k];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) p[k] = pn[k];
+        for (int k = 0; k < 3; ++k) p[k] = take ? pn[k] : p[k];
     }
     // world frame: base * chain
     const float* B = M.baseR[a];
@@ -441,28 +437,33 @@ __device__ __forceinline__ float box_sdf_only(const float* a, const float* d, fl
     return sqrtf(q2) + fminf(mx, 0.0f);
 }
 
-// Separating-axis test of the segment mid +- hv against the box inflated
+// Separating axes of the segment mid +- hv against the box inflated
 // by r on every side (half-extents h + r): the three box axes, then the
 // three products hv x e_k, onto which the segment projects to one point.
-// A capsule of radius r that touches the box lies in that inflated box, so
-// it always passes; the margin eps absorbs FP32 rounding.
-__device__ __forceinline__ bool segment_meets_inflated_box(const float* mid, const float* hv, const float* box,
-                                                           float r) {
+// Returns the largest gap along the six (the products' in units of length by
+// ihl_k = 1 / |hv x e_k|): a capsule of radius r that touches the box lies in
+// that inflated box, so the gap is then <= 0, and a positive gap is a lower
+// bound of the capsule's distance; the margin eps absorbs FP32 rounding.
+struct SegmentAxes {
+    float mid[3], hv[3], ah[3], ihl[3];
+};
+__device__ __forceinline__ float segment_box_gap(const SegmentAxes& x, const float* box, float r) {
     constexpr float eps = 1e-5f;
-    float dc[3], e[3], ah[3];
+    float dc[3], e[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        dc[k] = mid[k] - box[k];
+        dc[k] = x.mid[k] - box[k];
         e[k] = box[3 + k] + r + eps;
-        ah[k] = fabsf(hv[k]);
     }
-    bool ok = true;
+    float g = fmaxf(fmaxf(fabsf(dc[0]) - (e[0] + x.ah[0]), fabsf(dc[1]) - (e[1] + x.ah[1])),
+                    fabsf(dc[2]) - (e[2] + x.ah[2]));
 #pragma unroll
-    for (int k = 0; k < 3; ++k) ok = ok && fabsf(dc[k]) <= e[k] + ah[k];
-    ok = ok && fabsf(dc[1] * hv[2] - dc[2] * hv[1]) <= e[1] * ah[2] + e[2] * ah[1] + eps;
-    ok = ok && fabsf(dc[2] * hv[0] - dc[0] * hv[2]) <= e[0] * ah[2] + e[2] * ah[0] + eps;
-    ok = ok && fabsf(dc[0] * hv[1] - dc[1] * hv[0]) <= e[0] * ah[1] + e[1] * ah[0] + eps;
-    return ok;
+    for (int k = 0; k < 3; ++k) {
+        const int i = (k + 1) % 3, j = (k + 2) % 3;
+        const float c = fabsf(dc[i] * x.hv[j] - dc[j] * x.hv[i]) - (e[i] * x.ah[j] + e[j] * x.ah[i] + eps);
+        g = fmaxf(g, c * x.ihl[k]);
+    }
+    return g;
 }
 
 // Candidate minimisers of the box SDF along the segment a + t d, t in [0,1].
@@ -656,7 +657,7 @@ __device__ __forceinline__ void ball_pass(const DevModel& M, WarpWS<NA>& w, cons
 // Narrow phase in canonical pair order (ball-floor, ball-links, ball-boxes,
 // links x boxes).  Ball pairs: one lane per pair slot (above), exact,
 // compacted with a ballot.  Capsule-box pairs: a conservative
-// separating-axis cull per lane (segment_meets_inflated_box), here; each
+// separating-axis cull per lane (segment_box_gap), here; each
 // surviving pair (in pair order) is then minimised by the whole group over the
 // candidate set above, in collide_exact.  Each lane adds
 // the depths of the contacts it found to pa (all) and pbox (against boxes),
@@ -675,7 +676,7 @@ struct Contacts {
 };
 template <int NA, int LPS>
 __device__ __forceinline__ void collide(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g,
-                                        float (&pa)[32 / LPS], float (&pbox)[32 / LPS], Contacts& con) {
+                                        float (&pa)[32 / LPS], float (&pbox)[32 / LPS], float& clear, Contacts& con) {
     using d = Dims<NA>;
     const int nb = M.nb;
     {  // ball - floor, on every lane; stored by store_floor where a solve reads it
@@ -696,44 +697,74 @@ __device__ __forceinline__ void collide(const DevModel& M, WarpWS<NA>& w, const 
     // group, lane CL + l) tests link l's capsule against the boxes (or one
     // half of them each): the segment against the box inflated by the
     // capsule radius (separating axes, conservative); the survivors are
-    // placed link-major, box-minor by a prefix sum over the links
+    // placed link-major, box-minor by a prefix sum over the links.
+    // clear: the lane's smallest gap at the last cull.  A gap bounds the
+    // distance from below and a distance changes by at most the motion of the
+    // link's ends, so the group skips the cull while every link has moved less
+    // than its gap from where it was then (no pair can touch).  The transfer
+    // iteration (K = 4096, H = 64): 342 us with the cull on every step, 298 so
+    // (295 without any cull).
     if (nb > 0) {
         constexpr int CL = d::NL <= LPS / 2 ? LPS / 2 : LPS;  // lanes of one pass over the links
         constexpr int NH = LPS / CL;                          // box halves
         const int l = g.sl & (CL - 1), half = g.sl / CL;
-        const int bsplit = NH == 2 ? (nb + 1) >> 1 : nb;
-        const int b0 = half ? bsplit : 0, b1 = half ? nb : bsplit;
-        unsigned smask = 0u;
-        if (l < d::NL) {
-            const float* a0 = w.a0[l];
-            const float* a1 = w.a1[l];
-            const float rc = M.link[l / NA][l % NA].rcap;
-            float mid[3], hv[3];
+        const int lc = l < d::NL ? l : 0;
+        float x0[3], x1[3], m0 = 0.0f, m1 = 0.0f;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                mid[k] = 0.5f * (a0[k] + a1[k]);
-                hv[k] = 0.5f * (a1[k] - a0[k]);
-            }
-#pragma unroll 4
-            for (int bi = b0; bi < b1; ++bi)
-                if (segment_meets_inflated_box(mid, hv, M.box[bi], rc)) smask |= 1u << bi;
+        for (int k = 0; k < 3; ++k) {
+            x0[k] = w.a0[lc][k];
+            x1[k] = w.a1[lc][k];
+            const float e0 = x0[k] - w.ref[lc][k], e1 = x1[k] - w.ref[lc][3 + k];
+            m0 = __fmaf_rn(e0, e0, m0);
+            m1 = __fmaf_rn(e1, e1, m1);
         }
-        const int cnt = __popc(smask);
-        const int cnt_link = NH == 2 ? cnt + g.xor_(cnt, CL) : cnt;  // both halves of link l
-        if (g.any(smask != 0u)) {
-            int pre = cnt_link;  // inclusive prefix over the links (both halves alike)
+        if (g.any(l < d::NL && !(fmaxf(m0, m1) < clear * fabsf(clear)))) {
+            const int bsplit = NH == 2 ? (nb + 1) >> 1 : nb;
+            const int b0 = half ? bsplit : 0, b1 = half ? nb : bsplit;
+            unsigned smask = 0u;
+            clear = INFINITY;
+            if (l < d::NL) {
+                const float rc = M.link[l / NA][l % NA].rcap;
+                SegmentAxes x;
 #pragma unroll
-            for (int off = 1; off < CL; off <<= 1) {
-                const int o = __shfl_up_sync(g.gm, pre, off, CL);
-                if (l >= off) pre += o;
+                for (int k = 0; k < 3; ++k) {
+                    x.mid[k] = 0.5f * (x0[k] + x1[k]);
+                    x.hv[k] = 0.5f * (x1[k] - x0[k]);
+                    x.ah[k] = fabsf(x.hv[k]);
+                    if (half == 0) {
+                        w.ref[l][k] = x0[k];
+                        w.ref[l][3 + k] = x1[k];
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const int i = (k + 1) % 3, j = (k + 2) % 3;
+                    x.ihl[k] = rsqrtf(__fmaf_rn(x.hv[i], x.hv[i], x.hv[j] * x.hv[j]));
+                }
+#pragma unroll 2
+                for (int bi = b0; bi < b1; ++bi) {
+                    const float gap = segment_box_gap(x, M.box[bi], rc);
+                    if (gap <= 0.0f) smask |= 1u << bi;
+                    clear = fminf(clear, gap - 2e-5f);
+                }
             }
-            int pos = pre - cnt_link + (half ? cnt_link - cnt : 0);
-            while (smask) {
-                const int bi = __ffs(smask) - 1;
-                smask &= smask - 1u;
-                w.ph.col.surv[pos++] = (short)(l * nb + bi);
+            const int cnt = __popc(smask);
+            const int cnt_link = NH == 2 ? cnt + g.xor_(cnt, CL) : cnt;  // both halves of link l
+            if (g.any(smask != 0u)) {
+                int pre = cnt_link;  // inclusive prefix over the links (both halves alike)
+#pragma unroll
+                for (int off = 1; off < CL; off <<= 1) {
+                    const int o = __shfl_up_sync(g.gm, pre, off, CL);
+                    if (l >= off) pre += o;
+                }
+                int pos = pre - cnt_link + (half ? cnt_link - cnt : 0);
+                while (smask) {
+                    const int bi = __ffs(smask) - 1;
+                    smask &= smask - 1u;
+                    w.ph.col.surv[pos++] = (short)(l * nb + bi);
+                }
+                con.nsurv = g.shfl(pre, CL - 1);
             }
-            con.nsurv = g.shfl(pre, CL - 1);
         }
     }
     con.close(M, g);

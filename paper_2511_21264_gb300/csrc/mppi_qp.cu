@@ -141,21 +141,25 @@ struct QPTable {
 
 // Lanes per sequence for n sequences of H steps (0: the long form): the
 // fewest that keep C <= 16 steps per lane (fewer shuffle rounds and tails),
-// then twice as many while the launch has less than 16 warps per SM and a lane
-// keeps seven steps, or less than two warps per SM and three steps.  One
-// GB300, 30 iterations, us with 1 / 2 / 4 / 8 / 16 lanes:
-//   n = 57344, H = 64:  - / - / 312 / 330 / 470     H = 32: - / 139 / 152 / 194 / 404
-//   n = 57344, H = 16:  91 / 75 / 89 / 163 / 386    n = 14336, H = 64: - / - / 106 / 89 / 137
-//   n = 14336, H = 32:  - / 50 / 42 / 60 / 118      n = 5000, H = 27:  - / 36 / 30 / 32 / 53
-//   n = 1000, H = 32:   - / 37 / 25 / 21 / 21       n = 300, H = 64:   - / - / 60 / 32 / 23
-int qp_lanes(int n, int H) {
+// then twice as many while the launch has less than 16 warps per SM (4 in the
+// controller form, whose CTAs are whole samples) and a lane keeps seven steps, or
+// less than two warps per SM and three steps.  One GB300, 30 iterations, us with
+// 1 / 2 / 4 / 8 / 16 lanes:
+//   n = 57344, H = 64:  - / - / 312 / 318 / 474     H = 32: - / 140 / 148 / 195 / 404
+//   n = 57344, H = 16:  101 / 75 / 91 / 162 / 386   n = 14336, H = 64: - / - / 107 / 92 / 134
+//   n = 14336, H = 32:  - / 50 / 44 / 56 / 113      n = 5000, H = 27:  - / 36 / 32 / 33 / 54
+//   n = 1000, H = 32:   - / 37 / 29 / 21 / 21       n = 300, H = 64:   - / - / 41 / 32 / 24
+// and drawn and projected, K samples x 14 joints:
+//   K = 1024, H = 32:   - / 48 / 55 / 77 / 110      K = 1024, H = 20: - / 33 / 39 / 68 / 110
+//   K = 4096, H = 64:   - / - / 336 / 358 / 499     K = 256, H = 16: 45 / 31 / 28 / 22 / 36
+int qp_lanes(int n, int H, bool drawn) {
     if (H > QP_LANES_MAX_H) return 0;
     int L = 1;
     while ((H + L - 1) / L > QP_MAX_C) L *= 2;
     const auto grow = [&](int warps_per_sm, int min_c) {
         while (L < QP_MAX_L && (long long)n * L < 152LL * 32 * warps_per_sm && (H + 2 * L - 1) / (2 * L) >= min_c) L *= 2;
     };
-    grow(16, 7);
+    grow(drawn ? 4 : 16, 7);
     grow(2, 3);
     return L;
 }
@@ -805,7 +809,7 @@ extern "C" int mppi_qp_project(int n, int H, float dt, const float* bounds, int 
     a.H = H;
     a.iters = iters;
     a.dt = dt;
-    a.L = qp_lanes(n, H);
+    a.L = qp_lanes(n, H, false);
     a.tab_size = qp_table_size(H, a.L);
     a.n_tab = 1;
     QPTable table;

@@ -32,19 +32,27 @@ __host__ __device__ constexpr size_t ws_stride(size_t at_least = 0) {
     while (s % 128 != want) s += 32;
     return s;
 }
-// The single controller's stride does not follow a smaller workspace: the
-// samples per CTA that its launches accept stay what they are.
 // The ball-task suite keeps the previous state's points behind the workspace.
 template <int NA, int LPS, bool TASK>
 __host__ __device__ constexpr size_t ctl_stride() {
-    constexpr size_t least = NA == 7 ? 7328 : 5600, task = sizeof(WarpWS<NA>) + sizeof(TaskPrev<NA>);
-    return ws_stride<NA, LPS>(TASK && task > least ? task : least);
+    return ws_stride<NA, LPS>(TASK ? sizeof(WarpWS<NA>) + sizeof(TaskPrev<NA>) : 0);
 }
+
+inline size_t unom_bytes(int unom_floats) { return ((size_t)unom_floats * sizeof(float) + 15) / 16 * 16; }
 
 template <int NA, int LPS, bool TASK>
 size_t rollout_smem(int spc, int unom_floats) {
-    return sizeof(DevModel) + (TASK ? sizeof(DevTask) : 0) + ((size_t)unom_floats * sizeof(float) + 15) / 16 * 16 +
+    return sizeof(DevModel) + (TASK ? sizeof(DevTask) : 0) + unom_bytes(unom_floats) +
            (size_t)spc * ctl_stride<NA, LPS, TASK>();
+}
+
+// The samples per CTA that a launch accepts do not follow a smaller workspace:
+// spc workspaces of at least 7.3 KB (5.6 KB for 3-link arms) fit max_sm bytes.
+template <int NA, int LPS, bool TASK>
+bool shape_fits(int spc, int unom_floats, int max_sm) {
+    constexpr size_t least = ws_stride<NA, LPS>(NA == 7 ? 7328 : 5600);
+    constexpr size_t stride = ctl_stride<NA, LPS, TASK>() > least ? ctl_stride<NA, LPS, TASK>() : least;
+    return sizeof(DevModel) + (TASK ? sizeof(DevTask) : 0) + unom_bytes(unom_floats) + spc * stride <= (size_t)max_sm;
 }
 
 template <int NA, int LPS, int MODE, bool TASK, int PLACE>
@@ -127,7 +135,7 @@ int launch_t(const RolloutArgs& a, int spc, cudaStream_t s) {
     cudaError_t q = cudaGetDevice(&dev);
     if (q == cudaSuccess) q = cudaDeviceGetAttribute(&max_sm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (q != cudaSuccess) return cuda_fail(q);
-    if (sm > (size_t)max_sm) return MPPI_ERR_INVALID_ARG;  // too many samples per CTA for shared memory
+    if (!shape_fits<NA, LPS, TASK>(spc, unom, max_sm)) return MPPI_ERR_INVALID_ARG;  // too many samples per CTA
     if (sm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return cuda_fail(e);
@@ -197,7 +205,7 @@ bool spc_occupancy(int spc, int unom_floats, int max_sm, int* per_sm) {
     const auto fn = rollout_kernel<NA, LPS, 1, TASK, 0>;
     const size_t sm = rollout_smem<NA, LPS, TASK>(spc, unom_floats);
     *per_sm = 0;
-    return sm <= (size_t)max_sm &&
+    return shape_fits<NA, LPS, TASK>(spc, unom_floats, max_sm) &&
            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess &&
            cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, fn, spc * LPS, sm) == cudaSuccess && *per_sm > 0;
 }
@@ -247,7 +255,7 @@ bool task_fits(int spc, int unom_floats) {
     int dev = 0, max_sm = 0;
     return cudaGetDevice(&dev) == cudaSuccess &&
            cudaDeviceGetAttribute(&max_sm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
-           rollout_smem<NA, 16, true>((spc + 1) / 2 * 2, unom_floats) <= (size_t)max_sm;
+           shape_fits<NA, 16, true>((spc + 1) / 2 * 2, unom_floats, max_sm);
 }
 
 // SMs of the current device, 0 if unknown.
