@@ -466,6 +466,26 @@ __device__ __forceinline__ float segment_box_gap(const SegmentAxes& x, const flo
     return g;
 }
 
+// The same test alone, where no gap is kept: whether no axis separates.
+__device__ __forceinline__ bool segment_meets_inflated_box(const float* mid, const float* hv, const float* box,
+                                                           float r) {
+    constexpr float eps = 1e-5f;
+    float dc[3], e[3], ah[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        dc[k] = mid[k] - box[k];
+        e[k] = box[3 + k] + r + eps;
+        ah[k] = fabsf(hv[k]);
+    }
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ok = ok && fabsf(dc[k]) <= e[k] + ah[k];
+    ok = ok && fabsf(dc[1] * hv[2] - dc[2] * hv[1]) <= e[1] * ah[2] + e[2] * ah[1] + eps;
+    ok = ok && fabsf(dc[2] * hv[0] - dc[0] * hv[2]) <= e[0] * ah[2] + e[2] * ah[0] + eps;
+    ok = ok && fabsf(dc[0] * hv[1] - dc[1] * hv[0]) <= e[0] * ah[1] + e[1] * ah[0] + eps;
+    return ok;
+}
+
 // Candidate minimisers of the box SDF along the segment a + t d, t in [0,1].
 // The SDF is convex along the segment and piecewise smooth; its minimum lies
 // at an end point, at a slab-plane or axis-centre crossing (kinks), at the
@@ -676,7 +696,8 @@ struct Contacts {
 };
 template <int NA, int LPS>
 __device__ __forceinline__ void collide(const DevModel& M, WarpWS<NA>& w, const Lanes<LPS>& g,
-                                        float (&pa)[32 / LPS], float (&pbox)[32 / LPS], float& clear, Contacts& con) {
+                                        float (&pa)[32 / LPS], float (&pbox)[32 / LPS], float& clear, bool last,
+                                        Contacts& con) {
     using d = Dims<NA>;
     const int nb = M.nb;
     {  // ball - floor, on every lane; stored by store_floor where a solve reads it
@@ -703,7 +724,9 @@ __device__ __forceinline__ void collide(const DevModel& M, WarpWS<NA>& w, const 
     // link's ends, so the group skips the cull while every link has moved less
     // than its gap from where it was then (no pair can touch).  The transfer
     // iteration (K = 4096, H = 64): 342 us with the cull on every step, 298 so
-    // (295 without any cull).
+    // (295 without any cull).  last: no step follows, so no gap is formed
+    // (single steps of 16384 transfer states 34.8 -> 32.8 us; a constant false
+    // where the samples are drawn, whose rollouts are long).
     if (nb > 0) {
         constexpr int CL = d::NL <= LPS / 2 ? LPS / 2 : LPS;  // lanes of one pass over the links
         constexpr int NH = LPS / CL;                          // box halves
@@ -741,11 +764,17 @@ __device__ __forceinline__ void collide(const DevModel& M, WarpWS<NA>& w, const 
                     const int i = (k + 1) % 3, j = (k + 2) % 3;
                     x.ihl[k] = rsqrtf(__fmaf_rn(x.hv[i], x.hv[i], x.hv[j] * x.hv[j]));
                 }
+                if (last) {
+#pragma unroll 4
+                    for (int bi = b0; bi < b1; ++bi)
+                        if (segment_meets_inflated_box(x.mid, x.hv, M.box[bi], rc)) smask |= 1u << bi;
+                } else {
 #pragma unroll 2
-                for (int bi = b0; bi < b1; ++bi) {
-                    const float gap = segment_box_gap(x, M.box[bi], rc);
-                    if (gap <= 0.0f) smask |= 1u << bi;
-                    clear = fminf(clear, gap - 2e-5f);
+                    for (int bi = b0; bi < b1; ++bi) {
+                        const float gap = segment_box_gap(x, M.box[bi], rc);
+                        if (gap <= 0.0f) smask |= 1u << bi;
+                        clear = fminf(clear, gap - 2e-5f);
+                    }
                 }
             }
             const int cnt = __popc(smask);

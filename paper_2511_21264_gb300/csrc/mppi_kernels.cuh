@@ -134,7 +134,7 @@ __device__ __forceinline__ float rollout_sample(const DevModel& M, WarpWS<NA>& w
         // from the kinematics are no longer live across it
         dynamics<NA>(M, w, g, io.err, Rl, cl, 0, false);
         Contacts con;
-        collide<NA>(M, w, g, pacc, pbacc, clear, con);
+        collide<NA>(M, w, g, pacc, pbacc, clear, MODE == 0 && h + 1 == io.H, con);
         g.sync();
         if (con.nsurv > 0) {
             n_exact += sl == 0 ? con.nsurv : 0;
