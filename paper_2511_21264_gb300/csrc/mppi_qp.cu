@@ -562,11 +562,12 @@ __device__ __forceinline__ float qp_scaled_row(float val, float& y, float lo, fl
     return rs * (w - y);
 }
 
-// ADMM iterations of one thread's sequence.  xb[t*T] = (x_{t+1}, (B^T vt)_{t+1})
-// on entry holds the start point x = prefix sums of vt; y[t*T] = 0.  On exit
-// xb[.].x holds the last iterate.
-__device__ void qp_long_admm(const QPClass& c, const float4* __restrict__ band, int H, int iters, float dt, float q,
-                        float qd, float2* xb, float4* yv, int T) {
+// ADMM iterations of one thread's sequence.  xs[t*T] = x_{t+1} on entry holds
+// the start point, the prefix sums of vt; y[t*T] = 0; rhs(t) = (B^T vt)_{t+1},
+// row(r) = row r of the band factor.  On exit xs holds the last iterate.
+template <class Row, class Rhs>
+__device__ __forceinline__ void qp_long_admm(const QPClass& c, const Row& row, const Rhs& rhs, int H, int iters, float dt,
+                                             float q, float qd, float* xs, float4* yv, int T) {
     const float s0 = c.s[0], s1 = c.s[1], s2 = c.s[2], s3 = c.s[3];
     const float rs0 = c.rho * s0, rs1 = c.rho * s1, rs2 = c.rho * s2, rs3 = c.rho * s3;
     float Plo, Phi, Vlo, Vhi, Alo, Ahi, A0lo, A0hi, Jlo, Jhi, J1lo, J1hi;
@@ -577,8 +578,6 @@ __device__ void qp_long_admm(const QPClass& c, const float4* __restrict__ band, 
     qp_bound(s2, c.lo[2] * dt + qd, c.hi[2] * dt + qd, A0lo, A0hi);  // v_{-1} = qd moved into the bounds
     qp_bound(s3, c.lo[3] * dt2, c.hi[3] * dt2, Jlo, Jhi);
     qp_bound(s3, c.lo[3] * dt2 - qd, c.hi[3] * dt2 - qd, J1lo, J1hi);
-    const float4* __restrict__ bf = band;      // forward rows
-    const float4* __restrict__ bb = band + H;  // backward rows
     // slot index i (0 <= i < H) of this thread's vectors and band rows;
     // checked in the bounds-check build, the identity otherwise
     auto sl = [H](int i) { return MPPI_IN_RANGE(i, H) ? i : 0; };
@@ -593,9 +592,8 @@ __device__ void qp_long_admm(const QPClass& c, const float4* __restrict__ band, 
         // substitution chain (the operations and their order are unchanged)
 #pragma unroll 4
         for (int t = 0; t < H; ++t) {
-            const float2 xv = xb[(size_t)sl(t) * T];
+            const float xp1 = xs[(size_t)sl(t) * T], bt = rhs(t);
             float4 y = yv[(size_t)sl(t) * T];
-            const float xp1 = xv.x;
             const float d1 = xp1 - x0, d2 = d1 - d1p, d3 = d2 - d2p;
             const float eP = qp_scaled_row(s0 * xp1, y.x, Plo, Phi, rs0);
             const float eV = qp_scaled_row(s1 * d1, y.y, Vlo, Vhi, rs1);
@@ -604,14 +602,14 @@ __device__ void qp_long_admm(const QPClass& c, const float4* __restrict__ band, 
             if (t >= 1) eJ = qp_scaled_row(s3 * d3, y.w, t == 1 ? J1lo : Jlo, t == 1 ? J1hi : Jhi, rs3);
             yv[(size_t)sl(t) * T] = y;
             // row t touches x_{t+1} (+1), x_t (-1, -2, -3), x_{t-1} (+1, +3), x_{t-2} (-1)
-            const float r3 = xv.y + eP + eV + eA + eJ;
+            const float r3 = bt + eP + eV + eA + eJ;
             r2 = r2 - eV - 2.0f * eA - 3.0f * eJ;
             r1 = r1 + eA + 3.0f * eJ;
             r0 = r0 - eJ;
             if (t >= 3) {  // x_{t-2} is complete: substitute (index i = t-2, slot t-3)
-                const float4 L = bf[sl(t - 3)];
+                const float4 L = row(sl(t - 3));
                 const float z = (r0 - L.y * z1 - L.z * z2 - L.w * z3) * L.x;
-                xb[(size_t)sl(t - 3) * T].x = z;
+                xs[(size_t)sl(t - 3) * T] = z;
                 z3 = z2;
                 z2 = z1;
                 z1 = z;
@@ -627,9 +625,9 @@ __device__ void qp_long_admm(const QPClass& c, const float4* __restrict__ band, 
         for (int i = H - 2; i <= H; ++i) {
             const float r = i == H - 2 ? r0 : (i == H - 1 ? r1 : r2);
             if (i < 1) continue;
-            const float4 L = bf[sl(i - 1)];
+            const float4 L = row(sl(i - 1));
             const float z = (r - L.y * z1 - L.z * z2 - L.w * z3) * L.x;
-            xb[(size_t)sl(i - 1) * T].x = z;
+            xs[(size_t)sl(i - 1) * T] = z;
             z3 = z2;
             z2 = z1;
             z1 = z;
@@ -638,8 +636,8 @@ __device__ void qp_long_admm(const QPClass& c, const float4* __restrict__ band, 
         float p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;  // x_{i+1}, x_{i+2}, x_{i+3}
 #pragma unroll 4
         for (int i = H; i >= 1; --i) {
-            const float4 L = bb[sl(i - 1)];
-            float* slot = &xb[(size_t)sl(i - 1) * T].x;
+            const float4 L = row(H + sl(i - 1));
+            float* slot = &xs[(size_t)sl(i - 1) * T];
             const float xi = (*slot - L.y * p1 - L.z * p2 - L.w * p3) * L.x;
             *slot = xi;
             p3 = p2;
@@ -667,49 +665,55 @@ __device__ __forceinline__ float qp_sample(const QPArgs& a, uint2 key, uint32_t 
     return v;
 }
 
-// Sequence i: class i / per_cls, member i % per_cls.
-// The standalone form (vin given) has its one class and table as parameters.
+// ALONE: the standalone form, sequence i of class `own` with the table as a
+// parameter: its rows are uniform reads of constant memory, which a chain of
+// dependent steps waits for less than for cached global ones (43,973 x 110,
+// 20 iterations: 1,259 -> 1,094 us; 1,335 x 106, 30 iterations: 370 -> 313).
+// Else sequence i = j K + k is sample k of joint (class) j, drawn here.
+template <bool ALONE>
 __global__ void __launch_bounds__(64) qp_long_kernel(QPArgs a, const __grid_constant__ QPClass own,
                                                      const __grid_constant__ QPTable table) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int T = blockDim.x, tid = threadIdx.x;
+    const int T = blockDim.x, tid = threadIdx.x, H = a.H;
     float4* yv = reinterpret_cast<float4*>(smem) + tid;
-    float2* xb = reinterpret_cast<float2*>(smem + (size_t)a.H * T * sizeof(float4)) + tid;
+    float* xs = reinterpret_cast<float*>(smem + (size_t)H * T * sizeof(float4)) + tid;
+    float* bs = xs + (size_t)H * T;  // B^T vt
     const int i = blockIdx.x * T + tid;
     if (i >= a.n) return;
-    const int cls = a.vin ? 0 : i / a.per_cls, mem = a.vin ? i : i % a.per_cls;
-    const QPClass c = a.vin ? own : a.cls[MPPI_IN_RANGE(cls, a.n_cls) ? cls : 0];
-    const float4* band = a.vin ? table.v : a.tab + (size_t)(a.n_tab > 1 ? cls : 0) * a.tab_size;
-    const long long nq = a.vin ? a.n : a.n_cls;
-    const float q = ld_checked(a.q0, a.vin ? i : cls, nq), qd = ld_checked(a.qd0, a.vin ? i : cls, nq);
-    auto sl = [&a](int h) { return MPPI_IN_RANGE(h, a.H) ? h : 0; };  // this thread's slots
-    // start point x = prefix sums of vt, and (B^T vt)_i = vt_{i-1} - vt_i (vt_H for i = H)
+    const int cls = ALONE ? 0 : i / a.per_cls, mem = ALONE ? i : i % a.per_cls;
+    const QPClass c = ALONE ? own : a.cls[MPPI_IN_RANGE(cls, a.n_cls) ? cls : 0];
+    const long long nq = ALONE ? a.n : a.n_cls;
+    const float q = ld_checked(a.q0, ALONE ? i : cls, nq), qd = ld_checked(a.qd0, ALONE ? i : cls, nq);
+    auto sl = [H](int h) { return MPPI_IN_RANGE(h, H) ? h : 0; };  // this thread's slots
+    auto rhs = [&](int t) { return bs[(size_t)sl(t) * T]; };
     uint2 key{};
     uint32_t iter = 0;
-    if (!a.vin) {
+    if (!ALONE) {
         key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
         iter = (uint32_t)(a.iter_ptr ? *a.iter_ptr : a.iter_val);
     }
+    // start point x = prefix sums of vt, and (B^T vt)_i = vt_{i-1} - vt_i (vt_H for i = H)
     float prev = 0.0f, acc = 0.0f;
-    for (int h = 0; h < a.H; ++h) {
-        float vt;
-        if (a.vin) {
-            vt = ld_checked(a.vin, (long long)i * a.H + h, a.in_n);
-        } else {  // sample k = member, joint j = class
-            vt = qp_sample(a, key, iter, mem, cls, h);
-        }
+    for (int h = 0; h < H; ++h) {
+        const float vt =
+            ALONE ? ld_checked(a.vin, (long long)i * H + h, a.in_n) : qp_sample(a, key, iter, mem, cls, h);
         acc += vt;
-        if (h > 0) xb[(size_t)sl(h - 1) * T].y = prev - vt;
-        xb[(size_t)sl(h) * T].x = acc;
+        if (h > 0) bs[(size_t)sl(h - 1) * T] = prev - vt;
+        xs[(size_t)sl(h) * T] = acc;
         yv[(size_t)sl(h) * T] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         prev = vt;
     }
-    xb[(size_t)sl(a.H - 1) * T].y = prev;
-    qp_long_admm(c, band, a.H, a.iters, a.dt, q, qd, xb, yv, T);
+    bs[(size_t)sl(H - 1) * T] = prev;
+    if (ALONE) {
+        qp_long_admm(c, [&](int r) { return table.v[r]; }, rhs, H, a.iters, a.dt, q, qd, xs, yv, T);
+    } else {
+        const float4* band = a.tab + (size_t)(a.n_tab > 1 ? cls : 0) * a.tab_size;
+        qp_long_admm(c, [&](int r) { return __ldg(&band[r]); }, rhs, H, a.iters, a.dt, q, qd, xs, yv, T);
+    }
     float xp = 0.0f;
-    for (int h = 0; h < a.H; ++h) {
-        const float x = xb[(size_t)sl(h) * T].x;
-        const long long o = a.vin ? (long long)i * a.H + h : ((long long)h * a.per_cls + mem) * a.nu + cls;
+    for (int h = 0; h < H; ++h) {
+        const float x = xs[(size_t)sl(h) * T];
+        const long long o = ALONE ? (long long)i * H + h : ((long long)h * a.per_cls + mem) * a.nu + cls;
         if (MPPI_IN_RANGE(o, a.out_n)) a.out[o] = x - xp;
         xp = x;
     }
@@ -737,25 +741,28 @@ int launch_c(const QPArgs& a, const QPClass* c, const QPTable* table, cudaStream
     return cudaGetLastError() == cudaSuccess ? MPPI_OK : MPPI_ERR_CUDA;
 }
 
-// 24 H bytes of shared memory per thread: 64 threads per CTA while that
-// stays within 100 KB (two CTAs per SM), else one warp.
+// 24 H bytes of shared memory per thread: 64 threads while they stay within
+// 100 KB (two CTAs per SM), else one warp.
+template <bool ALONE>
 int launch_long(const QPArgs& a, const QPClass* c, const QPTable* table, cudaStream_t s) {
-    const size_t per = (size_t)a.H * (sizeof(float4) + sizeof(float2));
+    const size_t per = (size_t)a.H * (sizeof(float4) + 2 * sizeof(float));
     const int T = 64 * per <= 100 * 1024 ? 64 : 32;
     const size_t sm = T * per;
     if (sm > 227 * 1024) return MPPI_ERR_UNSUPPORTED;
     static const QPClass no_class{};
     static const QPTable no_table{};
     if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(qp_long_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e =
+            cudaFuncSetAttribute(qp_long_kernel<ALONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return MPPI_ERR_CUDA;
     }
-    qp_long_kernel<<<(int)(((long long)a.n + T - 1) / T), T, sm, s>>>(a, c ? *c : no_class, table ? *table : no_table);
+    qp_long_kernel<ALONE>
+        <<<(int)(((long long)a.n + T - 1) / T), T, sm, s>>>(a, c ? *c : no_class, table ? *table : no_table);
     return cudaGetLastError() == cudaSuccess ? MPPI_OK : MPPI_ERR_CUDA;
 }
 
 int launch_any(const QPArgs& a, const QPClass* c, const QPTable* table, cudaStream_t s) {
-    if (a.L == 0) return launch_long(a, c, table, s);
+    if (a.L == 0) return table ? launch_long<true>(a, c, table, s) : launch_long<false>(a, c, table, s);
     switch ((a.H + a.L - 1) / a.L) {
         case 1: return launch_c<1>(a, c, table, s);
         case 2: return launch_c<2>(a, c, table, s);
