@@ -189,6 +189,7 @@ struct __align__(16) WarpWS {
             CArr<float, 2 * MAXL + 2> motion;                             // of each link's ends since the last state
             CArr<short, 2 * MAXL * MAXB + 2 * MAXL + MAXL * MAXL + 1> pair;  // in pair order; 0x4000: dist holds the previous one
             CArr<float, 2 * MAXL * MAXB + 2 * MAXL + MAXL * MAXL> dist;
+            CArr<float, NA * NA + 2 * NA> val;  // what the listed ball-link and link-link pairs add
         } task;
     } ph;
 };

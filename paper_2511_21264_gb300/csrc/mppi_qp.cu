@@ -21,10 +21,12 @@
 // precomputed 3 x 3 maps, and a correction (backward: three products per
 // step; forward: the pass again from the true state).  When L does not divide
 // H, slot 0 of the last lanes is empty; lane 0 is always full.
-// Bound: issue slots (72-79 warp instructions per 32 steps and iteration, 65-70%
-// of the slots) and, with the gains in shared memory, its 128-bit loads (four
-// wavefronts each even when the lanes share addresses): a shape's register
-// bound is set so that most gains stay in registers.  One GB300, 30 iterations:
+// Bound: at C = 16 the latency of two warps per scheduler (63-65 warp
+// instructions per 32 steps and iteration, 51-53% of the issue slots); with
+// more warps and the gains in shared memory the issue slots (72-79
+// instructions, 65-70%) and the 128-bit loads (four wavefronts each even when
+// the lanes share addresses), which is no faster: a shape's register bound is
+// set so that most gains stay in registers.  One GB300, 30 iterations:
 // 57344 x 64 takes 312 us against 676 with the long form below (one warp per
 // scheduler, 30% of the issue slots); 5000 x 27 takes 31 us against 38 with one
 // lane per step and a dense inverse; 1024 samples x 14 joints x 32 drawn and

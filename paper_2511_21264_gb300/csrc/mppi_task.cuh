@@ -23,13 +23,15 @@ struct __align__(16) DevTask {
 template <int NA, int LPS>
 struct TaskDims {
     static constexpr int CC = (2 * NA + NA * NA + LPS - 1) / LPS;  // passes of the second kind at most
+    // two passes or less cost no more than the screen (task_state)
+    static constexpr bool ALL = CC <= 2;
 };
 
 template <int NA, int LPS>
 struct TaskAcc {
     // lower bounds at the previous state: of this lane's link's distance to any
     // box, and of its pairs' distances in the passes -- the distance itself
-    // where the bit of exact is set
+    // where the bit of exact is set (or every pair forms it)
     float lbox, lb[TaskDims<NA, LPS>::CC];
     unsigned exact;
     float c[32 / LPS];              // barrier + penetration count, per slot of the pair list
@@ -272,7 +274,12 @@ __device__ __forceinline__ float quat_angle(const float* q, const float* qs) {
 // 2e-5 m) are far above the rounding of the distances, so the terms are those of
 // testing every pair.  One iteration of the transfer with the suite (K = 4096, H =
 // 64): 1,360 us with every distance on 32 lanes, 800 screened per pair (16
-// lanes), 525 with the bound per link.
+// lanes), 525 with the bound per link (485 since the box cull is skipped too).
+// Where the pairs of the second kind take two passes or less, every lane forms
+// its pairs' distances: on those few lanes' worth of pairs the list costs as
+// much as they do.  us per iteration with every distance / screened / so: lift
+// K = 1024, H = 32 139.5 / 143.8 / 134.2, planar K = 100, H = 20 83.7 / 89.0 /
+// 80.8, transfer (16 boxes) K = 1216, H = 32 317 / 160 / 153.
 template <int NA, int LPS>
 __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, WarpWS<NA>& w, const Lanes<LPS>& g,
                                            const float (&Rl)[9], bool first, TaskAcc<NA, LPS>& acc) {
@@ -309,9 +316,15 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
         for (int s = 0; s < CC; ++s) acc.lb[s] = g.sl + LPS * s < ncc ? segment_pair(g.sl + LPS * s, true) : 0.0f;
         acc.exact = ~0u;
     } else {
+        const auto need = [](float motion) { return __fmaf_rn(motion, 1.00001f, 2e-5f); };
+        const auto value = [keep](float d0, float d1) { return fmaxf(-d1 + keep * d0, 0.0f) + (d1 < 0.0f ? 1.0f : 0.0f); };
+        const unsigned below = (1u << g.sl) - 1u;
+        int nlist = 0;
+        bool tbox = false;  // this lane's link meets its bound
+        int pbox = 0;
         // motion of every link's ends and of the ball since the previous state
-        float ml = 0.0f;
-        if (own) {
+        float ml = 0.0f, mb = 0.0f;
+        if (own && !(TaskDims<NA, LPS>::ALL && nb == 0)) {
             float m0 = 0.0f, m1 = 0.0f;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
@@ -320,21 +333,17 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
                 m1 = __fmaf_rn(e1, e1, m1);
             }
             ml = sqrtf(fmaxf(m0, m1));
-            sc.motion[g.sl] = ml;
+            if (!TaskDims<NA, LPS>::ALL) sc.motion[g.sl] = ml;
         }
-        float mb = 0.0f;
+        if (!TaskDims<NA, LPS>::ALL) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const float e = w.q[d::B + k] - pv.ball[k];
-            mb = __fmaf_rn(e, e, mb);
+            for (int k = 0; k < 3; ++k) {
+                const float e = w.q[d::B + k] - pv.ball[k];
+                mb = __fmaf_rn(e, e, mb);
+            }
+            mb = sqrtf(mb);
+            g.sync();
         }
-        mb = sqrtf(mb);
-        g.sync();
-        const auto need = [](float motion) { return __fmaf_rn(motion, 1.00001f, 2e-5f); };
-        const unsigned below = (1u << g.sl) - 1u;
-        int nlist = 0;
-        bool tbox = false;  // this lane's link meets its bound
-        int pbox = 0;
         if (nb > 0) {
             const float nd = need(ml);
             tbox = own && !(nd <= T.gamma * acc.lbox);
@@ -348,68 +357,86 @@ __device__ __forceinline__ void task_state(const DevModel& M, const DevTask& T, 
         }
         const int nbox = nlist;
         unsigned trig = 0u;
+        if (!TaskDims<NA, LPS>::ALL) {
+#pragma unroll
+            for (int s = 0; s < CC; ++s) {
+                const int b = g.sl + LPS * s;
+                const bool in = b < ncc, ball = b < nball;
+                const int r = in && !ball ? b - nball : 0, i = r / NA, j = r - i * NA;
+                const float nd = need(ball ? sc.motion[in ? b : 0] + mb : sc.motion[i] + sc.motion[NA + j]);
+                const float lbv = acc.lb[s];
+                const bool t = in && !(nd <= T.gamma * lbv);
+                const unsigned m = g.ballot(t);
+                float nl = lbv - nd;
+                if (t) {
+                    const int pos = nlist + __popc(m & below);
+                    sc.pair[pos] = (short)(b | ((acc.exact >> s) & 1u ? 0x4000 : 0));
+                    sc.dist[pos] = lbv;
+                    nl = __int_as_float(pos);
+                    trig |= 1u << s;
+                }
+                acc.lb[s] = nl;
+                nlist += __popc(m);
+            }
+            acc.exact = trig;
+        }
+        if (nlist > 0) {
+            g.sync();
+            // entry e of the boxes' list adds to slot e % 32, whatever LPS is
+#pragma unroll 1
+            for (int e = g.sl; e < nbox; e += LPS) {
+                const int b = sc.pair[e], l = b / nb, bx = b - l * nb;
+                const float rc = M.link[l / NA][l % NA].rcap;
+                float d0 = 0.0f, d1 = 0.0f;
+#pragma unroll 1
+                for (int now = 0; now < 2; ++now) {  // one copy of the distance's code
+                    d1 = capsule_box_distance(now ? &w.a0[l][0] : &pv.a[l][0], now ? &w.a1[l][0] : &pv.a[l][3], rc,
+                                              M.box[bx]);
+                    d0 = now ? d0 : d1;
+                }
+                const float v = value(d0, d1);
+                const int ps = (e / LPS) & (PS - 1);
+#pragma unroll
+                for (int t = 0; t < PS; ++t) acc.c[t] += ps == t ? v : 0.0f;
+                sc.dist[e] = d1;
+            }
+            if (!TaskDims<NA, LPS>::ALL) {
+#pragma unroll 1
+                for (int e = nbox + ((g.sl - nbox) & (LPS - 1)); e < nlist; e += LPS) {
+                    const int en = sc.pair[e], b = en & 0x3fff;
+                    float d0 = sc.dist[e], d1 = 0.0f;
+#pragma unroll 1
+                    for (int now = en & 0x4000 ? 1 : 0; now < 2; ++now) {
+                        d1 = segment_pair(b, now != 0);
+                        d0 = now ? d0 : d1;
+                    }
+                    sc.dist[e] = d1;
+                    sc.val[e - nbox] = value(d0, d1);
+                }
+            }
+            g.sync();
+            // the listed pairs' distances back to their lanes
+            if (tbox) {
+                acc.lbox = INFINITY;
+                for (int bx = 0; bx < nb; ++bx) acc.lbox = fminf(acc.lbox, sc.dist[pbox + bx]);
+            }
+        }
+        // pair b of the second kind adds to slot b % 32, whatever LPS is
 #pragma unroll
         for (int s = 0; s < CC; ++s) {
             const int b = g.sl + LPS * s;
-            const bool in = b < ncc, ball = b < nball;
-            const int r = in && !ball ? b - nball : 0, i = r / NA, j = r - i * NA;
-            const float nd = need(ball ? sc.motion[in ? b : 0] + mb : sc.motion[i] + sc.motion[NA + j]);
-            const float lbv = acc.lb[s];
-            const bool t = in && !(nd <= T.gamma * lbv);
-            const unsigned m = g.ballot(t);
-            float nl = lbv - nd;
-            if (t) {
-                const int pos = nlist + __popc(m & below);
-                sc.pair[pos] = (short)(b | ((acc.exact >> s) & 1u ? 0x4000 : 0));
-                sc.dist[pos] = lbv;
-                nl = __int_as_float(pos);
-                trig |= 1u << s;
+            if (TaskDims<NA, LPS>::ALL) {
+                if (b < ncc) {
+                    const float d1 = segment_pair(b, true);
+                    acc.c[s & (PS - 1)] += value(acc.lb[s], d1);
+                    acc.lb[s] = d1;
+                }
+            } else if ((trig >> s) & 1u) {
+                const int pos = __float_as_int(acc.lb[s]);
+                acc.c[s & (PS - 1)] += sc.val[pos - nbox];
+                acc.lb[s] = sc.dist[pos];
             }
-            acc.lb[s] = nl;
-            nlist += __popc(m);
         }
-        acc.exact = trig;
-        g.sync();
-        // entry e of the list is slot e % 32's, whatever LPS is
-        auto add = [&](int e, float d0, float d1) {
-            const float v = fmaxf(-d1 + keep * d0, 0.0f) + (d1 < 0.0f ? 1.0f : 0.0f);
-            const int ps = (e / LPS) & (PS - 1);
-#pragma unroll
-            for (int t = 0; t < PS; ++t) acc.c[t] += ps == t ? v : 0.0f;
-            sc.dist[e] = d1;
-        };
-#pragma unroll 1
-        for (int e = g.sl; e < nbox; e += LPS) {
-            const int b = sc.pair[e], l = b / nb, bx = b - l * nb;
-            const float rc = M.link[l / NA][l % NA].rcap;
-            float d0 = 0.0f, d1 = 0.0f;
-#pragma unroll 1
-            for (int now = 0; now < 2; ++now) {  // one copy of the distance's code
-                d1 = capsule_box_distance(now ? &w.a0[l][0] : &pv.a[l][0], now ? &w.a1[l][0] : &pv.a[l][3], rc, M.box[bx]);
-                d0 = now ? d0 : d1;
-            }
-            add(e, d0, d1);
-        }
-#pragma unroll 1
-        for (int e = nbox + ((g.sl - nbox) & (LPS - 1)); e < nlist; e += LPS) {
-            const int en = sc.pair[e], b = en & 0x3fff;
-            float d0 = sc.dist[e], d1 = 0.0f;
-#pragma unroll 1
-            for (int now = en & 0x4000 ? 1 : 0; now < 2; ++now) {
-                d1 = segment_pair(b, now != 0);
-                d0 = now ? d0 : d1;
-            }
-            add(e, d0, d1);
-        }
-        g.sync();
-        // the listed pairs' distances back to their lanes
-        if (tbox) {
-            acc.lbox = INFINITY;
-            for (int bx = 0; bx < nb; ++bx) acc.lbox = fminf(acc.lbox, sc.dist[pbox + bx]);
-        }
-#pragma unroll
-        for (int s = 0; s < CC; ++s)
-            if ((trig >> s) & 1u) acc.lb[s] = sc.dist[__float_as_int(acc.lb[s])];
     }
     if (own) {
 #pragma unroll
