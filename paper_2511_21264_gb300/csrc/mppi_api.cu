@@ -904,7 +904,7 @@ static int launch_elite(mppi_ctx* c, const float* costs, const float* u_nom, flo
     // the register network (P <= 1024)
     const size_t sm = (size_t)(P <= 1024 ? 2048 : P) * sizeof(unsigned long long);
     if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(elite_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = open_shared_memory(elite_select_kernel, SMALL_STATIC_SMEM);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     // both kernels as programmatic dependents: their launches overlap the tails

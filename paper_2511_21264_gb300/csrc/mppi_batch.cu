@@ -238,17 +238,17 @@ int batch_shape_t(int spc, int lps, int place, int max_h, BatchLaunch* L) {
     const int max_unom = max_h * Dims<NA>::NU <= 2048 ? max_h * Dims<NA>::NU : 0;
     L->max_unom = max_unom;
     L->smem = sizeof(DevModel) + ((size_t)max_unom * sizeof(float) + 15) / 16 * 16 + (size_t)spc * batch_ws_stride<NA>(lps);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L->smem);
+    cudaError_t e = open_shared_memory(fn, SMALL_STATIC_SMEM);
     if (e != cudaSuccess) return MPPI_ERR_CUDA;
     int per_sm = 0, dev = 0, sms = 0;
     BatchFn fn0 = batch_fn<NA>(lps, 0, 0);  // the projected-sample form of the layout
-    if (fn0) e = cudaFuncSetAttribute(fn0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L->smem);
+    if (fn0) e = open_shared_memory(fn0, SMALL_STATIC_SMEM);
     if (e != cudaSuccess) return MPPI_ERR_CUDA;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, spc * lps, L->smem);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return MPPI_ERR_CUDA;
-    L->grid = (per_sm > 0 ? per_sm : 1) * sms;
+    if (e != cudaSuccess || per_sm <= 0) return MPPI_ERR_CUDA;
+    L->grid = per_sm * sms;
     L->spc = spc;
     L->lps = lps;
     L->place = place;
@@ -278,7 +278,7 @@ int launch_batch_iteration(const BatchInst* insts, int n, int ntiles, int nrows,
     if (L.sel_P > 0) {  // elite thresholds of the instances that use them
         const size_t sm = (size_t)(L.sel_P <= 1024 ? 2048 : L.sel_P) * sizeof(unsigned long long);
         if (sm > 48 * 1024) {
-            e = cudaFuncSetAttribute(batch_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            e = open_shared_memory(batch_select_kernel, SMALL_STATIC_SMEM);
             if (e != cudaSuccess) return MPPI_ERR_CUDA;
         }
         batch_select_kernel<<<n, 1024, sm, s>>>(insts, n);

@@ -26,6 +26,24 @@ constexpr int ERRB_TIMEOUT = 4;
 struct DevModel;
 struct DevTask;
 
+// Opens kernel fn for launches with as much dynamic shared memory as a CTA of
+// the current device can have beside fn's static_bytes.  The limit belongs to the
+// kernel, so every handle and thread that launches fn shares it: set to the size
+// of one launch it refused another's larger one (two batches of different
+// horizons in turn, two threads' projections of different lengths).  Always the
+// same value, so calls may overlap.
+template <class F>
+cudaError_t open_shared_memory(F* fn, int static_bytes = 0) {
+    int dev = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - static_bytes);
+    return e;
+}
+// static shared memory of the kernels that have some beside the dynamic block
+// (a few words; rounded up)
+constexpr int SMALL_STATIC_SMEM = 1024;
+
 struct HostModelInfo {
     int na = 0, nb = 0;
     std::vector<float> x0;

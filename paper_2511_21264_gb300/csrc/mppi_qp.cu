@@ -736,7 +736,7 @@ int launch_c(const QPArgs& a, const QPClass* c, const QPTable* table, cudaStream
     const size_t normals = (size_t)S * a.H * ((a.nu + 3) / 4), tabs = (size_t)a.n_tab * a.tab_size;
     const size_t sm = ((size_t)(S * a.nu * rs + 3) / 4 + std::max(normals, tabs)) * sizeof(float4);
     if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(qp_sample_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = open_shared_memory(qp_sample_kernel<C>);
         if (e != cudaSuccess) return MPPI_ERR_CUDA;
     }
     qp_sample_kernel<C><<<(a.per_cls + S - 1) / S, QP_MAX_L * a.nu, sm, s>>>(a);
@@ -754,8 +754,7 @@ int launch_long(const QPArgs& a, const QPClass* c, const QPTable* table, cudaStr
     static const QPClass no_class{};
     static const QPTable no_table{};
     if (sm > 48 * 1024) {
-        cudaError_t e =
-            cudaFuncSetAttribute(qp_long_kernel<ALONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = open_shared_memory(qp_long_kernel<ALONE>);
         if (e != cudaSuccess) return MPPI_ERR_CUDA;
     }
     qp_long_kernel<ALONE>

@@ -137,7 +137,7 @@ int launch_t(const RolloutArgs& a, int spc, cudaStream_t s) {
     if (q != cudaSuccess) return cuda_fail(q);
     if (!shape_fits<NA, LPS, TASK>(spc, unom, max_sm)) return MPPI_ERR_INVALID_ARG;  // too many samples per CTA
     if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = open_shared_memory(fn);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     const int grid = (a.n + spc - 1) / spc;
@@ -206,7 +206,7 @@ bool spc_occupancy(int spc, int unom_floats, int max_sm, int* per_sm) {
     const size_t sm = rollout_smem<NA, LPS, TASK>(spc, unom_floats);
     *per_sm = 0;
     return shape_fits<NA, LPS, TASK>(spc, unom_floats, max_sm) &&
-           cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess &&
+           open_shared_memory(fn) == cudaSuccess &&
            cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, fn, spc * LPS, sm) == cudaSuccess && *per_sm > 0;
 }
 
