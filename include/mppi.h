@@ -397,7 +397,8 @@ int mppi_batch_get_launch(const mppi_batch *b, int *samples_per_cta, int *order)
  * placement of the lone ball contact's solve (as mppi_set_layout).  A new
  * batch has the layout that its total number of samples gives a controller
  * (16 lanes with 2 or 16 samples per CTA, else 32 with 4) unless a tuned
- * choice is stored for it. */
+ * choice is stored for it; until the samples per CTA are set or tuned they
+ * follow the layout (4 in a layout that is not the default). */
 int mppi_batch_set_layout(mppi_batch *b, int lanes_per_sample, int placement);
 int mppi_batch_get_layout(const mppi_batch *b, int *lanes_per_sample, int *placement);
 /* Autotuner: times `reps` iterations of every shape -- lanes per sample

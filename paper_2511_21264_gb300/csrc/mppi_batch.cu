@@ -366,6 +366,8 @@ extern "C" int mppi_tune_store(const char* key, int spc, int order, int lps, int
 // ---------------------------------------------------------------------------
 struct mppi_batch {
     int n = 0, na = 0, nu = 0, max_h = 0, spc = 4, order = 1, lps = 32, place = 0;
+    long long ksum = 0;           // samples of all instances
+    bool spc_auto = true;         // spc is the library's choice for the layout
     std::vector<mppi_batch_desc> desc;
     std::vector<BatchInst> inst;  // per user instance
     std::vector<int> perm;        // execution order -> user instance
@@ -428,6 +430,19 @@ void build_order(mppi_batch* b) {
     }
     b->ntiles = t;
     b->nrows = r;
+}
+
+// Samples per CTA in layout lps when neither the caller nor the tuning table
+// sets them: where the samples take the 16-lane layout by default, the widest
+// CTAs once they fill every SM (32 each), else one-warp CTAs, which spread evenly;
+// 4 in every other layout (16 samples do not fit a CTA on 32 lanes).  One
+// GB300, ms: 64 controllers of the configurations' pool 7.3 on 32 lanes with 4
+// samples per CTA, 5.5 / 5.1 / 4.6 / 4.5 on 16 with 2 / 4 / 8 / 16; 5 controllers
+// (5632 samples) 0.45, and 0.31 / 0.32 / 0.30 / 0.28; 2 (3072 samples) 0.46, and
+// 0.44 / 0.51 / 0.51 / 0.49
+int default_batch_spc(const mppi_batch* b, int lps) {
+    if (lps != 16 || default_lps(b->na, b->ksum) != 16) return 4;
+    return b->ksum > 32LL * sm_count() ? 16 : 2;
 }
 
 int reshape(mppi_batch* b) {
@@ -593,23 +608,17 @@ int mppi_batch_create(const mppi_batch_desc* desc, int n, mppi_batch** out) {
     std::snprintf(key, sizeof key, "nv%d_nb%d_n%d_K%lld_H%d", 2 * na + 6, boxes <= 0 ? 0 : (boxes <= 8 ? 8 : 16), n,
                   ksum, b->max_h);
     b->key = key;
-    // without a stored choice: a single controller's layout for the batch's
-    // samples; on 16 lanes the widest CTAs once the samples fill every SM (32
-    // each), one-warp CTAs below, which spread evenly.  One GB300, ms: 64
-    // controllers of the configurations' pool 7.3 on 32 lanes with 4 samples per
-    // CTA, 5.5 / 5.1 / 4.6 / 4.5 on 16 with 2 / 4 / 8 / 16; 5 controllers (5632
-    // samples) 0.45, and 0.31 / 0.32 / 0.30 / 0.28; 2 (3072 samples) 0.46, and
-    // 0.44 / 0.51 / 0.51 / 0.49
-    if (default_lps(na, ksum) == 16) {
-        b->lps = 16;
-        b->spc = ksum > 32LL * sm_count() ? 16 : 2;
-    }
+    // without a stored choice: a single controller's layout for the batch's samples
+    b->ksum = ksum;
+    b->lps = default_lps(na, ksum);
+    b->spc = default_batch_spc(b, b->lps);
     int spc = 0, order = 0, lps = 0, place = 0;
     if (mppi_tune_lookup(key, &spc, &order, &lps, &place) == MPPI_OK) {
         b->spc = spc;
         b->order = order;
         b->lps = lps;
         b->place = place;
+        b->spc_auto = false;
     }
     b->d_eq8.assign(n, nullptr);
     b->d_sel.assign(n, nullptr);
@@ -733,6 +742,8 @@ int mppi_batch_set_launch(mppi_batch* b, int spc, int order) {
         b->spc = os;
         b->order = oo;
         reshape(b);
+    } else if (spc != os) {
+        b->spc_auto = false;  // the default shape given back with another order stays the library's choice
     }
     return rc;
 }
@@ -749,6 +760,7 @@ int mppi_batch_set_layout(mppi_batch* b, int lps, int place) {
     if (lps == 0) lps = 32;
     if ((lps != 8 && lps != 16 && lps != 32) || place < 0 || place > 1) return MPPI_ERR_INVALID_ARG;
     const int ol = b->lps, op = b->place, os = b->spc;
+    if (b->spc_auto && lps != b->lps) b->spc = default_batch_spc(b, lps);
     b->lps = lps;
     b->place = place;
     const int rc = reshape(b);
@@ -930,6 +942,7 @@ int mppi_batch_autotune(mppi_batch* b, const float* const* states, float* const*
     b->order = bo;
     b->lps = bl;
     b->place = bp;
+    b->spc_auto = false;
     if (rc == MPPI_OK) rc = reshape(b);
     // the tuning iterations do not count: restore the counters
     if (rc == MPPI_OK) {
