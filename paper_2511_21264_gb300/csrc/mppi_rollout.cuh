@@ -199,7 +199,13 @@ int dispatch_rollout(int mode, const RolloutArgs& a, int spc, cudaStream_t s) {
 // fewest waves of CTAs over the SMs; within one wave the fewest samples on
 // the busiest SM, then the larger CTA (fewer model copies to stage; on
 // GB300 a 28-sample CTA per SM beat two 14-sample CTAs by 5%); past one wave
-// the most samples resident per SM, then the smaller CTA.
+// the most samples resident per SM, then the smaller CTA.  A load of
+// five warps of 7-link arms counts as six: a scheduler has two of them either
+// way, and in iterations whose launches overlap two five-warp CTAs come to share
+// SMs while others idle.  One GB300, us, 10 / 12 samples per CTA on 16 lanes:
+// K = 1217 transfer samples x 64 steps 249 / 208 per iteration (199 / 199 for the
+// rollout alone), K = 1500 lift x 32 120 / 100; 5 / 6 on 32 lanes: K = 650 transfer
+// 213 / 171, lift 106 / 86.
 template <int NA, int LPS, bool TASK>
 bool spc_occupancy(int spc, int unom_floats, int max_sm, int* per_sm) {
     const auto fn = rollout_kernel<NA, LPS, 1, TASK, 0>;
@@ -238,7 +244,8 @@ int choose_spc(int lps, int K, int unom_floats, bool task) {
         const long waves = (blocks + cap - 1) / cap;
         // lower is better: one wave -> load on the busiest SM (ties to the
         // larger CTA below); more -> minus the samples resident per SM
-        const long key = waves == 1 ? (blocks + nsm - 1) / nsm * spc : -(long)per_sm * spc;
+        long key = waves == 1 ? (blocks + nsm - 1) / nsm * spc : -(long)per_sm * spc;
+        if (NA == 7 && key == 5 * spw) key = 6 * spw;
         const bool tie_larger = waves == 1;
         if (waves < best_w || (waves == best_w && (key < best_key || (key == best_key && tie_larger)))) {
             best_w = waves;
@@ -271,9 +278,10 @@ inline int sm_count() {
 // take more than 8 warps per SM (7-link arms; 16 for the shorter 3-link steps,
 // where 32-lane groups can no longer hold all samples at once), else 32 (the
 // shorter per-step chain of one sample per warp).  One GB300, us per iteration
-// on 32 / 16 lanes: transfer H = 64, K = 1216 205 / 242, K = 2048 284 / 246,
-// K = 2432 288 / 270; lift H = 32, K = 1216 89 / 90, K = 2048 128 / 102;
-// planar H = 20, K = 2048 125 / 126, K = 4096 236 / 151.
+// on 32 / 16 lanes: transfer H = 64, K = 1216 180 / 193, K = 1217 215 / 208,
+// K = 1824 224 / 210, K = 2432 260 / 227; lift H = 32, K = 1216 91 / 88, K = 1217
+// 108 / 99, K = 2048 129 / 100; planar H = 20, K = 2048 138 / 135, K = 2500
+// 220 / 144, K = 4096 277 / 167.
 inline int default_lps(int na, long long K) {
     const int nsm = sm_count();
     return nsm > 0 && K > (na == 7 ? 8LL : 16LL) * nsm ? 16 : 32;

@@ -1,0 +1,47 @@
+"""The default layout and shape of a controller is no slower than the same
+controller on 32 lanes (the other layout of its range): us per iteration, both
+timed in turn, medians of 7 x 20 iterations.  Between 8 and 16 samples per SM,
+where the rules choose 16 lanes or the ball-task suite leaves them.  The bound
+of 1.08 is twice the spread of such medians (under 3%) and far below what a
+wrong choice costs there (1.11 and more)."""
+import numpy as np
+import pytest
+
+from paper_2511_21264_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+DEV = "cuda:0"
+
+
+def _time(ctl, x, u, out):
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    a.record()
+    for _ in range(20):
+        ctl.step(x, u, out)
+    b.record()
+    b.synchronize()
+    return a.elapsed_time(b) / 20
+
+
+def _ratio(scene, task, K, H):
+    from paper_2511_21264_gb300 import native
+    sc = scenes.dh_scene(seed=0, n_boxes=8 if scene == "transfer" else 0, task=scene)
+    m = native.Model(sc.to_blob())
+    x, u = torch.tensor(m.home(), device=DEV), torch.zeros((H, sc.nu), device=DEV)
+    out = torch.empty_like(u)
+    ctls = [native.Controller(m, K, H, 2.0, sc.sigma_vec(), 7) for _ in range(2)]
+    ctls[1].set_layout(32, 0)
+    for c in ctls:
+        if task is not None:
+            c.set_task_cost(scenes.ball_task(sc, task))
+        for _ in range(20):
+            c.step(x, u, out)
+    t = np.array([[_time(c, x, u, out) for c in ctls] for _ in range(7)])
+    assert all(c.sync() == 0 for c in ctls)
+    return np.median(t[:, 0]) / np.median(t[:, 1])
+
+
+@pytest.mark.parametrize("scene,K,H", [("transfer", 1300, 64), ("lift", 1500, 32)])
+def test_default_shape(scene, K, H):
+    assert _ratio(scene, None, K, H) <= 1.08
