@@ -344,7 +344,8 @@ int mppi_set_launch(mppi_ctx *c, int samples_per_cta);
  * solve of a lone ball contact with static geometry: 0 = fused with the
  * arms' factorisation (every lane runs both chains), 1 = after it.  Every
  * layout gives bitwise the same samples, costs and updates.  The ball-task
- * cost suite runs on 32 lanes where 8 are set, and with the fused placement.  Errors:
+ * cost suite runs on 32 lanes where 8 are set (and, with 7-link arms, up to
+ * 12 samples per SM until a layout is set), and with the fused placement.  Errors:
  * MPPI_ERR_INVALID_ARG for other values or more than 512 threads per CTA,
  * MPPI_ERR_UNSUPPORTED for 8 lanes with 7-link arms. */
 int mppi_set_layout(mppi_ctx *c, int lanes_per_sample, int placement);

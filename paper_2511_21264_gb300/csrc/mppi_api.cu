@@ -264,6 +264,7 @@ struct mppi_ctx {
     const mppi_model* m = nullptr;
     int K = 0, H = 0, spc = 4;
     int lps = 32, place = 0;  // lanes per sample, placement of the lone ball contact's solve
+    bool lps_auto = true;     // lps is the library's choice for the samples
     bool spc_auto = true;     // spc is the library's choice for the layout
     int spc_task = 0, spc_task_lps = 0;  // the ball-task suite's default shape in layout spc_task_lps
     float lambda = 1.0f;
@@ -422,13 +423,15 @@ static int default_spc(const mppi_ctx* c) { return default_spc_for(c, c->lps, fa
 
 // Layout and samples per CTA of a rollout: the handle's.  The ball-task suite
 // needs a lane per link and its own points in shared memory: it runs on 32
-// lanes where the handle has 8, and with its own default shape; a shape that the
-// caller chose is kept, on 32 lanes (at most 512 threads) where it does not fit.
+// lanes where the handle has 8, and with its own default layout and shape; a
+// layout or shape that the caller chose is kept, on 32 lanes (at most 512
+// threads) where the shape does not fit.
 static int rollout_shape(mppi_ctx* c, RolloutArgs* a) {
     a->lps = c->lps;
     a->place = c->place;
     if (!a->task) return c->spc;
     a->place = 0;
+    if (c->lps_auto) a->lps = default_lps(c->m->info.na, c->K, true);
     if (c->lps == 8) a->lps = 32;
     if (c->spc_auto) {
         if (c->spc_task_lps != a->lps) {
@@ -684,8 +687,9 @@ int mppi_set_layout(mppi_ctx* c, int lps, int place) {
     if ((lps != 8 && lps != 16 && lps != 32) || place < 0 || place > 1) return MPPI_ERR_INVALID_ARG;
     if (lps == 8 && c->m->info.na != 3) return MPPI_ERR_UNSUPPORTED;  // a 7-link arm needs 8 lanes per arm
     if (!c->spc_auto && c->spc * lps > 512) return MPPI_ERR_INVALID_ARG;
-    if (lps != c->lps || place != c->place) drop_graph(c);
+    if (c->lps_auto || lps != c->lps || place != c->place) drop_graph(c);
     c->lps = lps;
+    c->lps_auto = false;
     c->place = place;
     if (c->spc_auto) c->spc = default_spc(c);  // the default shape follows the layout
     return MPPI_OK;

@@ -282,9 +282,13 @@ inline int sm_count() {
 // K = 1824 224 / 210, K = 2432 260 / 227; lift H = 32, K = 1216 91 / 88, K = 1217
 // 108 / 99, K = 2048 129 / 100; planar H = 20, K = 2048 138 / 135, K = 2500
 // 220 / 144, K = 4096 277 / 167.
-inline int default_lps(int na, long long K) {
+// The ball-task suite forms every pair's distance on 32 lanes but screens the
+// pairs on 16, which costs more per step: 16 lanes from 12 samples per SM on
+// (H = 32, us on 32 / 16 lanes: transfer K = 1217 172 / 192, K = 1824 181 / 196, K =
+// 2048 198 / 195, K = 2500 299 / 222; lift 161 / 176, 171 / 180, 187 / 180, 280 / 205).
+inline int default_lps(int na, long long K, bool task = false) {
     const int nsm = sm_count();
-    return nsm > 0 && K > (na == 7 ? 8LL : 16LL) * nsm ? 16 : 32;
+    return nsm > 0 && K > (na == 7 ? (task ? 12LL : 8LL) : 16LL) * nsm ? 16 : 32;
 }
 
 int launch_rollout_na7(int mode, const RolloutArgs& a, int spc, cudaStream_t s);

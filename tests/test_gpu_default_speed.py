@@ -45,3 +45,8 @@ def _ratio(scene, task, K, H):
 @pytest.mark.parametrize("scene,K,H", [("transfer", 1300, 64), ("lift", 1500, 32)])
 def test_default_shape(scene, K, H):
     assert _ratio(scene, None, K, H) <= 1.08
+
+
+@pytest.mark.parametrize("K", [1300, 1500])
+def test_default_shape_of_the_ball_task_suite(K):
+    assert _ratio("transfer", 1, K, 32) <= 1.08
