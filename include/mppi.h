@@ -397,7 +397,7 @@ int mppi_batch_get_launch(const mppi_batch *b, int *samples_per_cta, int *order)
 /* Layout: lanes per sample (32, 16, or 8 for 3-link arms; 0 = 32) and the
  * placement of the lone ball contact's solve (as mppi_set_layout).  A new
  * batch has the layout that its total number of samples gives a controller
- * (16 lanes with 2 or 16 samples per CTA, else 32 with 4) unless a tuned
+ * (16 lanes with 2, 14 or 16 samples per CTA, else 32 with 4) unless a tuned
  * choice is stored for it; until the samples per CTA are set or tuned they
  * follow the layout (4 in a layout that is not the default). */
 int mppi_batch_set_layout(mppi_batch *b, int lanes_per_sample, int placement);

@@ -433,16 +433,20 @@ void build_order(mppi_batch* b) {
 }
 
 // Samples per CTA in layout lps when neither the caller nor the tuning table
-// sets them: where the samples take the 16-lane layout by default, the widest
-// CTAs once they fill every SM (32 each), else one-warp CTAs, which spread evenly;
-// 4 in every other layout (16 samples do not fit a CTA on 32 lanes).  One
-// GB300, ms: 64 controllers of the configurations' pool 7.3 on 32 lanes with 4
-// samples per CTA, 5.5 / 5.1 / 4.6 / 4.5 on 16 with 2 / 4 / 8 / 16; 5 controllers
-// (5632 samples) 0.45, and 0.31 / 0.32 / 0.30 / 0.28; 2 (3072 samples) 0.46, and
-// 0.44 / 0.51 / 0.51 / 0.49
+// sets them: where the samples take the 16-lane layout by default and fill every
+// SM, 16, or 14 where the staged nominal of a long horizon leaves an SM no room
+// for two CTAs of 16; with fewer samples one-warp CTAs, which spread evenly; 4 in
+// every other layout (16 samples do not fit a CTA on 32 lanes).  One GB300, ms: 4
+// controllers of 2048 transfer samples on 32 lanes with 4 samples per CTA, and on
+// 16 with 4 / 8 / 10 / 12 / 14 / 16: H = 64 0.92, 0.69 / 0.69 / 0.65 / 0.68 / 0.61 /
+// 0.60; H = 100 1.43, 1.06 / 1.06 / 1.00 / 1.05 / 0.93 / 1.31; H = 146 2.06, 1.53 /
+// 1.54 / 1.67 / 1.51 / 1.34 / 1.89.
 int default_batch_spc(const mppi_batch* b, int lps) {
+    const int nsm = sm_count();
     if (lps != 16 || default_lps(b->na, b->ksum) != 16) return 4;
-    return b->ksum > 32LL * sm_count() ? 16 : 2;
+    if (b->ksum <= 32LL * nsm) return 2;
+    BatchLaunch L{};
+    return batch_shape(b->na, 16, lps, 0, b->max_h, &L) == MPPI_OK && L.grid >= 2 * nsm ? 16 : 14;
 }
 
 int reshape(mppi_batch* b) {

@@ -40,3 +40,24 @@ def test_every_layout_after_creation(tmp_path, monkeypatch, cfg, K):
     b.set_launch(4, 1)
     b.set_layout(32, 1)
     assert b.get_launch()[0] == 4
+
+
+@pytest.mark.parametrize("cfg,H,spc", [(3, 64, 16), (3, 100, 14), (3, 146, 14), (3, 147, 16), (1, 100, 16)])
+def test_default_shape_keeps_two_ctas_on_an_sm(tmp_path, monkeypatch, cfg, H, spc):
+    # 6720 bytes a sample of the 7-link arms, 2608 the model, 1 KB reserved and,
+    # up to 2048 values, the staged nominal sequence: two CTAs of 16 samples fit
+    # an SM's 228 KB up to H = 99, two of 14 up to 146
+    monkeypatch.setenv("MPPI_TUNE_FILE", str(tmp_path / "none.txt"))
+    from paper_2511_21264_gb300 import native
+    sc = scenes.config(cfg)
+    K = 1300
+    m = native.Model(sc.to_blob())
+    b = native.Batch([(m, K, H, 1.0, sc.sigma_vec(), s) for s in range(4)])
+    assert (b.get_layout()[0], b.get_launch()[0]) == (16, spc)
+    x, us = torch.tensor(m.home(), device=DEV), [torch.zeros((H, sc.nu), device=DEV) for _ in range(4)]
+    b.step([x] * 4, us)
+    assert b.sync()[0] == 0
+    ctl = native.Controller(m, K, H, 1.0, sc.sigma_vec(), 2)
+    u = torch.zeros((H, sc.nu), device=DEV)
+    ctl.step(x, u)
+    assert ctl.sync() == 0 and torch.equal(u, us[2])
