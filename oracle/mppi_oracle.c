@@ -681,6 +681,10 @@ static void quat_mul(const double *a, const double *b, double *o) {
     o[0] = w; o[1] = x; o[2] = y; o[3] = z;
 }
 
+/* One Gauss-Seidel update of a row with diagonal den = A + R; a row that no
+ * coordinate moves (planar arms across their plane: den = 0) takes no impulse. */
+static double row_update(double lam, double res, double den) { return den == 0.0 ? 0.0 : lam - res / den; }
+
 /* x = (q, qd) -> x_out after one step of dt with controls u (nu).
  * Optionally returns the impulses (3 per contact) and the contacts. */
 int or_step_ex(const or_model *m, const double *x, const double *u, double *xo, or_step_info *info,
@@ -777,7 +781,7 @@ int or_step_ex(const or_model *m, const double *x, const double *u, double *xo, 
                 /* normal row */
                 double res = b[in] + R[in] * lam[in] - vstar[in];
                 for (int s = 0; s < nr; s++) res += A[in * nr + s] * lam[s];
-                double ln = lam[in] - res / (A[in * nr + in] + R[in]);
+                double ln = row_update(lam[in], res, A[in * nr + in] + R[in]);
                 lam[in] = ln > 0.0 ? ln : 0.0;
                 /* tangent rows, jointly, then the friction disk */
                 double rt[2];
@@ -787,8 +791,8 @@ int or_step_ex(const or_model *m, const double *x, const double *u, double *xo, 
                     for (int s = 0; s < nr; s++) acc += A[it * nr + s] * lam[s];
                     rt[tr] = acc;
                 }
-                double l1 = lam[in + 1] - rt[0] / (A[(in + 1) * nr + in + 1] + R[in + 1]);
-                double l2 = lam[in + 2] - rt[1] / (A[(in + 2) * nr + in + 2] + R[in + 2]);
+                double l1 = row_update(lam[in + 1], rt[0], A[(in + 1) * nr + in + 1] + R[in + 1]);
+                double l2 = row_update(lam[in + 2], rt[1], A[(in + 2) * nr + in + 2] + R[in + 2]);
                 double nrm = sqrt(l1 * l1 + l2 * l2), lim = m->mu * lam[in];
                 if (nrm > lim) {
                     double sc = nrm > 0.0 ? lim / nrm : 0.0;

@@ -1628,7 +1628,8 @@ __device__ __forceinline__ void contacts(const DevModel& M, WarpWS<NA>& w, const
                 w.G[(9 * q + 3 * k + m) * MAXC + c] = gv;
             }
         }
-        w.ph.con.iA[r] = 1.0f / gd;
+        // a row that no joint moves (planar arms across their plane) takes no impulse
+        w.ph.con.iA[r] = gd == 0.0f ? 0.0f : 1.0f / gd;
         float b4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int q = 0; q < d::NV; ++q) {
