@@ -59,6 +59,55 @@ struct CArr {
     __host__ __device__ __forceinline__ operator const T*() const { return v; }
 };
 
+// n elements of dynamic shared memory.  In the bounds-check build an array whose
+// operator[] checks the index; else the plain pointer (a wrapper changes how the
+// compiler allots the registers of kernels at their limit).
+#ifdef MPPI_BOUNDS_CHECK
+template <class T>
+struct Run {
+    T* p;
+    int n;
+    __device__ __forceinline__ Run(T* at, int len) : p(at), n(len) {}
+    template <class U>
+    __device__ __forceinline__ Run(const Run<U>& r) : p(r.p), n(r.n) {}
+    __device__ __forceinline__ T& operator[](int i) const {
+        if ((unsigned)i >= (unsigned)n) {
+            bounds_fail(BOUNDS_SHARED);
+            return *reinterpret_cast<T*>(g_bounds_sink);
+        }
+        return p[i];
+    }
+};
+template <class T>
+__device__ __forceinline__ Run<T> make_run(T* p, int n) {
+    return {p, n};
+}
+// the elements first .. first + len - 1, or all from first on
+template <class T>
+__device__ __forceinline__ Run<T> sub_run(Run<T> r, int first, int len) {
+    if (first < 0 || len < 0 || first + len > r.n) {
+        bounds_fail(BOUNDS_SHARED);
+        return {r.p, 0};
+    }
+    return {r.p + first, len};
+}
+template <class T>
+__device__ __forceinline__ Run<T> sub_run(Run<T> r, int first) {
+    return {r.p + first, r.n > first ? r.n - first : 0};
+}
+#else
+template <class T>
+using Run = T*;
+template <class T>
+__device__ __forceinline__ T* make_run(T* p, int) {
+    return p;
+}
+template <class T>
+__device__ __forceinline__ T* sub_run(T* r, int first, int = 0) {
+    return r + first;
+}
+#endif
+
 // True when 0 <= i < n; in the bounds-check build a false result also sets
 // the global-buffer bit.  Use as `if (MPPI_IN_RANGE(i, n)) p[i] = ...` or
 // around a read whose fallback keeps the lane's value.

@@ -300,7 +300,7 @@ __device__ __forceinline__ float qp_row(float val, float& y, float lo, float hi)
 }
 
 // acc += m x, m the rows at t[0], t[L], t[2 L]
-__device__ __forceinline__ void qp_map(const float4* t, int L, const float (&x)[3], float (&acc)[3]) {
+__device__ __forceinline__ void qp_map(Run<const float4> t, int L, const float (&x)[3], float (&acc)[3]) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const float4 m = t[i * L];
@@ -310,9 +310,9 @@ __device__ __forceinline__ void qp_map(const float4* t, int L, const float (&x)[
 
 // ADMM iterations of one sequence held by L consecutive lanes of a warp, this
 // one (p) with the C slots v (the input on entry, the last iterate on exit;
-// slot 0 unused when `empty`).  T: the table, lane p's entries at T + p.
+// slot 0 unused when `empty`).  T: the table, lane p's entries from p on.
 template <int C>
-__device__ __forceinline__ void qp_admm(const QPClass& c, const float4* T, int L, int p, bool empty, int iters, float dt,
+__device__ __forceinline__ void qp_admm(const QPClass& c, Run<const float4> T, int L, int p, bool empty, int iters, float dt,
                                         float q, float qd, float (&v)[C]) {
     const float idt = 1.0f / dt, dt2 = dt * dt;
     const float Plo = (c.lo[0] - q) * idt, Phi = (c.hi[0] - q) * idt, Vlo = c.lo[1], Vhi = c.hi[1];
@@ -321,9 +321,7 @@ __device__ __forceinline__ void qp_admm(const QPClass& c, const float4* T, int L
     const float rJ = c.rho * c.s[3] * c.s[3], rJ2 = -2.0f * rJ;
     const float on0 = empty ? 0.0f : 1.0f, onJ = empty || p == 0 ? 0.0f : 1.0f;  // slot 0's rows; step 0 has no jerk row
     const float qd0 = p == 0 ? qd : 0.0f;
-    const float4* kc = T + p;
-    const float4* psi = T + C * L + p;
-    const float4* maps = T + 2 * C * L + p;
+    const Run<const float4> kc = sub_run(T, p), psi = sub_run(T, C * L + p), maps = sub_run(T, 2 * C * L + p);
 
     float vt[C], P[C], y[4][C];
     // positions of the start point, and the two velocities before slot 0
@@ -393,8 +391,8 @@ __device__ __forceinline__ void qp_admm(const QPClass& c, const float4* T, int L
             d1 = dp;
         }
         float g[3] = {gP, g1, g2}, s[3];
-        const float4* mp = maps;
-        for (int off = 1; off < L; off <<= 1, mp += 6 * L) {
+        Run<const float4> mp = maps;
+        for (int off = 1; off < L; off <<= 1, mp = sub_run(mp, 6 * L)) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) s[k] = __shfl_down_sync(FULL, g[k], off, L);
             qp_map(mp, L, s, g);
@@ -417,8 +415,8 @@ __device__ __forceinline__ void qp_admm(const QPClass& c, const float4* T, int L
             st[2] = skip ? st[2] : st[1];
             st[1] = skip ? st[1] : x;
         }
-        mp = maps + 3 * L;
-        for (int off = 1; off < L; off <<= 1, mp += 6 * L) {
+        mp = sub_run(maps, 3 * L);
+        for (int off = 1; off < L; off <<= 1, mp = sub_run(mp, 6 * L)) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) s[k] = __shfl_up_sync(FULL, st[k], off, L);
             qp_map(mp, L, s, st);
@@ -450,19 +448,18 @@ __device__ __forceinline__ int qp_row_stride(int H) { return H | 1; }
 
 // The CTA's sequences from the stage through the iterations and back.
 template <int C>
-__device__ __forceinline__ void qp_solve(const QPArgs& a, const QPClass& c, const float4* T, float* row, int p, float q,
-                                         float qd) {
+__device__ __forceinline__ void qp_solve(const QPArgs& a, const QPClass& c, Run<const float4> T, Run<float> row, int p,
+                                         float q, float qd) {
     const int full = a.H - a.L * (C - 1);  // lanes with C steps; the others leave slot 0 empty
     const bool empty = p >= full;
     const int t0 = p * C - (empty ? p - full + 1 : 0);  // step of slot 0
-    auto at = [&a](int t) { return MPPI_IN_RANGE(t, a.H) ? t : 0; };
     float v[C];
 #pragma unroll
-    for (int i = 0; i < C; ++i) v[i] = i == 0 && empty ? 0.0f : row[at(t0 + i)];
+    for (int i = 0; i < C; ++i) v[i] = i == 0 && empty ? 0.0f : row[t0 + i];
     qp_admm<C>(c, T, a.L, p, empty, a.iters, a.dt, q, qd, v);
 #pragma unroll
     for (int i = 0; i < C; ++i)
-        if (!(i == 0 && empty)) row[at(t0 + i)] = v[i];
+        if (!(i == 0 && empty)) row[t0 + i] = v[i];
 }
 
 // Standalone form: one class, the table as a kernel parameter.
@@ -472,8 +469,9 @@ __global__ void __launch_bounds__(QP_THREADS, C <= 4 ? 6 : C <= 8 ? 4 : C <= 12 
     extern __shared__ __align__(16) float4 qsm[];
     const int tid = threadIdx.x, L = a.L, p = tid & (L - 1), seqs = QP_THREADS / L, rs = qp_row_stride(a.H);
     const int nt = a.tab_size;
-    float* stage = reinterpret_cast<float*>(qsm + nt);
-    for (int t = tid; t < nt; t += QP_THREADS) qsm[t] = table.v[t];
+    const Run<float4> tab = make_run(qsm, nt);
+    const Run<float> stage = make_run(reinterpret_cast<float*>(qsm + nt), seqs * rs);
+    for (int t = tid; t < nt; t += QP_THREADS) tab[t] = table.v[MPPI_IN_RANGE(t, QP_MAX_TABLE) ? t : 0];
     const long long i0 = (long long)blockIdx.x * seqs;
     const int ns = (int)(a.n - i0 < seqs ? a.n - i0 : seqs);  // sequences of this CTA
     const int lane = tid & 31, warp = tid >> 5;
@@ -483,7 +481,7 @@ __global__ void __launch_bounds__(QP_THREADS, C <= 4 ? 6 : C <= 8 ? 4 : C <= 12 
     __syncthreads();
     const int sq = tid / L;
     const long long i = i0 + (sq < ns ? sq : ns - 1);
-    qp_solve<C>(a, c, qsm, stage + sq * rs, p, ld_checked(a.q0, i, a.n), ld_checked(a.qd0, i, a.n));
+    qp_solve<C>(a, c, tab, sub_run(stage, sq * rs, a.H), p, ld_checked(a.q0, i, a.n), ld_checked(a.qd0, i, a.n));
     __syncthreads();
     for (int r = warp; r < ns; r += QP_THREADS / 32)
         for (int t = lane; t < a.H; t += 32)
@@ -500,23 +498,24 @@ __global__ void __launch_bounds__(224, C <= 4 ? 3 : C <= 8 ? 2 : 1) qp_sample_ke
     const int tid = threadIdx.x, T = blockDim.x, L = a.L, p = tid & (L - 1), S = QP_MAX_L / L, nu = a.nu, H = a.H;
     const int rs = qp_row_stride(H), k0 = blockIdx.x * S, nb = (nu + 3) / 4;
     const int ns = a.per_cls - k0 < S ? a.per_cls - k0 : S;  // samples of this CTA
-    float* stage = reinterpret_cast<float*>(qsm);
-    float4* tab = qsm + ((S * nu * rs + 3) >> 2);
-    float* z = reinterpret_cast<float*>(tab);
+    const Run<float> stage = make_run(reinterpret_cast<float*>(qsm), S * nu * rs);
+    float4* const after = qsm + ((S * nu * rs + 3) >> 2);
+    const Run<float4> draws = make_run(after, S * H * nb), tab = make_run(after, a.n_tab * a.tab_size);
+    const Run<float> z = make_run(reinterpret_cast<float*>(after), 4 * S * H * nb);
     const uint2 key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
     const uint32_t iter = (uint32_t)(a.iter_ptr ? *a.iter_ptr : a.iter_val);
     for (int b = tid; b < S * H * nb; b += T) {
         const int s = b / (H * nb), h = b / nb - s * H, jb = b % nb;
         float z4[4];
         block_normals4(philox4x32_10(make_uint4((uint32_t)jb, (uint32_t)h, (uint32_t)(k0 + s), iter), key), z4);
-        tab[b] = make_float4(z4[0], z4[1], z4[2], z4[3]);
+        draws[b] = make_float4(z4[0], z4[1], z4[2], z4[3]);
     }
     __syncthreads();
     const int jt = tid % nu;  // 16 nu threads: a thread stays with its joint
     for (int e = tid / nu; e < S * H; e += QP_MAX_L) {
         // the value the rollout's sampler draws, unclamped
         const int j = jt, s = e / H, h = e - s * H;
-        const float* zr = z + e * 4 * nb;
+        const Run<float> zr = sub_run(z, e * 4 * nb, 4 * nb);
         float v = ld_checked(a.u_nom, (long long)h * nu + j, (long long)H * nu);
         if (a.Lfac) {
             const long long r0 = ((long long)h * nu + j) * nu, n_l = (long long)H * nu * nu;
@@ -531,7 +530,7 @@ __global__ void __launch_bounds__(224, C <= 4 ? 3 : C <= 8 ? 2 : 1) qp_sample_ke
     __syncthreads();
     const int sq = tid / L, j = sq % nu;
     const QPClass c = a.cls[MPPI_IN_RANGE(j, a.n_cls) ? j : 0];
-    qp_solve<C>(a, c, tab + (a.n_tab > 1 ? j * a.tab_size : 0), stage + sq * rs, p, ld_checked(a.q0, j, a.n_cls),
+    qp_solve<C>(a, c, sub_run(tab, a.n_tab > 1 ? j * a.tab_size : 0, a.tab_size), sub_run(stage, sq * rs, H), p, ld_checked(a.q0, j, a.n_cls),
                 ld_checked(a.qd0, j, a.n_cls));
     __syncthreads();
     const int i = tid % (S * nu);  // L rows of S nu values at a time
