@@ -234,7 +234,11 @@ int mppi_best_controls(mppi_ctx *c, float *U_best, void *stream);
  *   q0, qd0  device, n floats: each sequence's present position, velocity
  *   v_in     device, n x H; v_out device, n x H (may alias v_in)
  * 1 <= H <= MPPI_QP_MAX_H, iters >= 0, rho > 0, dt > 0.  One kernel launch;
- * nothing is allocated or copied (the factors travel as its parameters). */
+ * nothing is allocated or copied (the factors travel as its parameters).
+ * Up to 80 steps the number of lanes that share a sequence follows from n and H,
+ * and so does the order of its sums: in a call of another n a sequence's result
+ * may differ by rounding (2e-6 of its 2-norm); above 80 steps it has the same
+ * bits.  A controller's projected samples depend on K in the same way. */
 int mppi_qp_project(int n, int H, float dt, const float *bounds, int iters, float rho, const float *scales,
                     const float *q0, const float *qd0, const float *v_in, float *v_out, void *stream);
 /* Turn the projection on inside the controller's iteration (iters > 0) or

@@ -145,7 +145,11 @@ struct QPTable {
 // fewest that keep C <= 16 steps per lane (fewer shuffle rounds and tails),
 // then twice as many while the launch has less than 16 warps per SM (4 in the
 // controller form, whose CTAs are whole samples) and a lane keeps seven steps, or
-// less than two warps per SM and three steps.  One GB300, 30 iterations, us with
+// less than two warps per SM and three steps.  So lanes of a shared sequence
+// hold at least two steps.  The 152 SMs of a GB300 are a constant here, not the
+// device's count: the split orders the sums, so a result follows from n and H
+// alone (one split for every n would cost 38% at n = 1000, H = 32, 33% at n = 300,
+// H = 64).  One GB300, 30 iterations, us with
 // 1 / 2 / 4 / 8 / 16 lanes:
 //   n = 57344, H = 64:  - / - / 312 / 318 / 474     H = 32: - / 140 / 148 / 195 / 404
 //   n = 57344, H = 16:  101 / 75 / 91 / 162 / 386   n = 14336, H = 64: - / - / 107 / 92 / 134
@@ -344,7 +348,10 @@ __device__ __forceinline__ void qp_admm(const QPClass& c, Run<const float4> T, i
     for (int i = 0; i < C; ++i) P[i] += pre;
     float x1, x2;
     {
-        // last two velocities of the lanes before (a lane may hold one step)
+        // last two velocities of the lanes before; the case of a lane with one
+        // step is for any split (qp_lanes makes none: without it, the compiler
+        // spills 96 bytes of 16 steps per lane instead of 12, and 4096 samples x 64
+        // take 652 us an iteration instead of 603)
         float l1 = v[C - 1], l2 = C > 1 ? v[C > 1 ? C - 2 : 0] : 0.0f;
         const bool one = C == 1 || (C == 2 && empty);
         float a1 = __shfl_up_sync(FULL, l1, 1, L), a2 = __shfl_up_sync(FULL, l2, 1, L);

@@ -248,7 +248,8 @@ def qp_project(v_in, bounds, q0, qd0, dt: float, iters: int = 30, rho: float = 1
                stream=None):
     """QP smoothing projection (Eq. 5) of n sequences (CUDA n x H) sharing
     one set of bounds (8 host values: lo, hi for position, velocity,
-    acceleration, jerk); q0, qd0: CUDA n present positions and velocities."""
+    acceleration, jerk); q0, qd0: CUDA n present positions and velocities.
+    Up to H = 80 a sequence's rounding depends on n (2e-6 of its 2-norm)."""
     n, H = v_in.shape
     v_out = v_in if v_out is None else v_out
     b = _host_f32(bounds, 8)
