@@ -27,10 +27,10 @@
 // instructions, 65-70%) and the 128-bit loads (four wavefronts each even when
 // the lanes share addresses), which is no faster: a shape's register bound is
 // set so that most gains stay in registers.  One GB300, 30 iterations:
-// 57344 x 64 takes 312 us against 676 with the long form below (one warp per
+// 57344 x 64 takes 312-319 us against 676 with the long form below (one warp per
 // scheduler, 30% of the issue slots); 5000 x 27 takes 31 us against 38 with one
 // lane per step and a dense inverse; 1024 samples x 14 joints x 32 drawn and
-// projected 55 us against 92.
+// projected 48 us against 92.
 //
 // Longer horizons: one thread per sequence, in the coordinates
 //   x_i = sum_{t<i} v_t   (i = 1..H, the position offset over dt),

@@ -46,8 +46,9 @@ size_t rollout_smem(int spc, int unom_floats) {
            (size_t)spc * ctl_stride<NA, LPS, TASK>();
 }
 
-// The samples per CTA that a launch accepts do not follow a smaller workspace:
-// spc workspaces of at least 7.3 KB (5.6 KB for 3-link arms) fit max_sm bytes.
+// The samples per CTA that a launch accepts do not follow a smaller workspace (what
+// the entry points refused stays refused): spc workspaces of at least 7.3 KB (5.6 KB
+// for 3-link arms) fit max_sm bytes.
 template <int NA, int LPS, bool TASK>
 bool shape_fits(int spc, int unom_floats, int max_sm) {
     constexpr size_t least = ws_stride<NA, LPS>(NA == 7 ? 7328 : 5600);
@@ -172,8 +173,8 @@ int launch_task(int mode, const RolloutArgs& a, int spc, cudaStream_t s) {
 
 // Launch for one arm size.  a.lps (0 = 32) and a.place select the layout;
 // spc is rounded up to whole warps.  The ball-task suite runs on 32 or 16
-// lanes per sample with the fused placement only.  A shape whose workspaces do not
-// fit one CTA's shared memory is refused with MPPI_ERR_INVALID_ARG.
+// lanes per sample with the fused placement only.  A shape that shape_fits turns
+// down is refused with MPPI_ERR_INVALID_ARG.
 template <int NA>
 int dispatch_rollout(int mode, const RolloutArgs& a, int spc, cudaStream_t s) {
     using namespace rollout_launch;
